@@ -657,7 +657,7 @@ int leanvec_search(lv_index *idx, const float *Q, int64_t m, const float *A, con
     if (params->event_begin) LV_CUDA(cudaEventRecord((cudaEvent_t)params->event_begin, st));
     if (mA == m) {
         rc = beam(p, st);
-        if (!rc && rerank) rc = launch_rerank(p, idx->num_sms, st);
+        if (!rc && rerank) rc = launch_rerank(p, st);
         if (rc) return rc;
     } else {
         BeamParams pa = p, pb = p;
@@ -676,8 +676,8 @@ int leanvec_search(lv_index *idx, const float *Q, int64_t m, const float *A, con
         LV_CUDA(cudaStreamWaitEvent(idx->aux, idx->ev_fork, 0));
         rc = beam(pa, st);
         if (!rc) rc = beam(pb, idx->aux);
-        if (!rc) rc = launch_rerank(pa, idx->num_sms, st);
-        if (!rc) rc = launch_rerank(pb, idx->num_sms, idx->aux);
+        if (!rc) rc = launch_rerank(pa, st);
+        if (!rc) rc = launch_rerank(pb, idx->aux);
         // join even after a failed launch, so that the caller's stream orders after the second one
         LV_CUDA(cudaEventRecord(idx->ev_join, idx->aux));
         LV_CUDA(cudaStreamWaitEvent(st, idx->ev_join, 0));

@@ -167,7 +167,7 @@ extern "C" int leanvec_search_noalloc(lv_index *idx, const float *Q, int64_t m, 
             break;
         }
         rc = launch_beam_search(idx, p, block, smem, st);
-        if (!rc && rerank) rc = launch_rerank(p, idx->num_sms, st);
+        if (!rc && rerank) rc = launch_rerank(p, st);
         if (rc) break;
         if (params->event_end && (e = cudaEventRecord((cudaEvent_t)params->event_end, st)) != cudaSuccess) {
             rc = cuda_fail(e, "search_noalloc: cudaEventRecord(event_end)");
