@@ -910,43 +910,37 @@ __global__ void __launch_bounds__(256, 3) beam_kernel(const BeamParams p) {
                 }
                 __syncwarp();
                 if (cv > 0) {
-                    // an id can appear twice in one round when two parents share a neighbour
-                    // that the visited cache did not catch (another warp's concurrent test, or a
-                    // forgotten id): keep the first copy
-                    bool anydup = false;
-                    if (Wr > 1) {
-                        if (cv <= 32) {
-                            // lanes past cv hold distinct negative keys that match nothing
-                            const int id = lane < cv ? cI[lane] : -2 - lane;
-                            const bool dup = (__match_any_sync(FULL, id) & lt) != 0u;
-                            if (dup) vPB[lane] = -1;
-                            anydup = __any_sync(FULL, dup);
-                        } else {
-                            bool d = false;
-                            for (int j = lane; j < cv; j += 32) {
-                                const int id = cI[j];
-                                bool dup = false;
-                                for (int u = 0; u < j; ++u) dup |= cI[u] == id;
-                                if (dup) {
-                                    vPB[j] = -1;
-                                    d = true;
-                                }
-                            }
-                            anydup = __any_sync(FULL, d);
+                    // rank of each candidate among the candidates; sPB[rank] = beam members ahead.  An id
+                    // can appear twice in one round when two parents share a neighbour that the visited
+                    // cache did not catch (another warp's concurrent test, or a forgotten id): its copies
+                    // have equal keys and share a rank, so the ranks add up to less than 0 + .. + cv - 1.
+                    // Only then are the copies looked for (the first one is kept) and the rest ranked again.
+                    for (;;) {
+                        unsigned ranks = 0;
+                        for (int j = lane; j < cv; j += 32) {
+                            const float s = cS[j];
+                            const int id = cI[j];
+                            int rank = 0;
+                            for (int u = 0; u < cv; ++u) rank += key_better(cS[u], cI[u], s, id) ? 1 : 0;
+                            const int pb = vPB[j] & 0xffff;
+                            sPB[rank] = pb;
+                            vPB[j] = pb | (rank << 16);
+                            ranks += (unsigned)rank;
                         }
-                        __syncwarp();
-                    }
-                    if (anydup) {
+                        if (Wr == 1 || __reduce_add_sync(FULL, ranks) == (unsigned)(cv * (cv - 1) / 2)) break;
                         int cv2 = 0;
                         for (int j0 = 0; j0 < cv; j0 += 32) {
                             const int j = j0 + lane;
-                            const bool keep = j < cv && vPB[j] >= 0;
+                            bool keep = j < cv;
                             float s = 0.f;
                             int id = 0, pb = 0;
                             if (keep) {
                                 s = cS[j];
                                 id = cI[j];
                                 pb = vPB[j];
+                                // copies before j: kept ones (already compacted) or of this chunk
+                                for (int u = 0; u < cv2; ++u) keep &= cI[u] != id;
+                                for (int u = j0; u < j; ++u) keep &= cI[u] != id;
                             }
                             const unsigned bal = __ballot_sync(FULL, keep);
                             __syncwarp();
@@ -959,17 +953,8 @@ __global__ void __launch_bounds__(256, 3) beam_kernel(const BeamParams p) {
                             cv2 += __popc(bal);
                             __syncwarp();
                         }
+                        if (cv2 == cv) break;  // equal ranks without copies: scores that do not order (NaN)
                         cv = cv2;
-                    }
-                    // rank of each candidate among the candidates; sPB[rank] = beam members ahead
-                    for (int j = lane; j < cv; j += 32) {
-                        const float s = cS[j];
-                        const int id = cI[j];
-                        int rank = 0;
-                        for (int u = 0; u < cv; ++u) rank += key_better(cS[u], cI[u], s, id) ? 1 : 0;
-                        const int pb = vPB[j];
-                        sPB[rank] = pb;
-                        vPB[j] = pb | (rank << 16);
                     }
                     __syncwarp();
                     // move beam members (in place, last chunk first; a member only moves right)
