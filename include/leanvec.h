@@ -395,9 +395,10 @@ typedef struct {
 typedef struct {
     lv_query_desc uniform;   /* used for every query when desc == NULL */
     int32_t projection;      /* lv_precision of the q -> A q GEMM */
-    int32_t hash_slots;      /* visited-cache slots per query (power of two; 0 = max(1024, 4 L) up to
-                                8192 slots of 32-bit ids, or twice as many 16-bit tags, see
-                                visited_bits) */
+    int32_t hash_slots;      /* visited-cache slots per query (power of two; 0 = the library's choice:
+                                max(1024, 4 L) up to 8192 slots of 32-bit ids; twice as many 16-bit
+                                tags with visited_bits 16; with visited_bits 0 as well, 2048 or 1024
+                                tags for long walks, see visited_bits) */
     int32_t warps_per_block; /* 0 = default */
     int32_t width;           /* search width: beam members expanded per round, 1..4 (0 = 1);
                                 width * R <= 256.  1 is the classic best-first traversal */
@@ -419,8 +420,11 @@ typedef struct {
                                 instructions per query; 2 holds 40 queries per SM instead of 24 and
                                 is faster when the index's primaries and graph sit in L2 and the
                                 batch spans several waves, 1 when they stream from DRAM */
-    int32_t visited_bits;     /* slot width of the visited cache of one query per warp: 32 (whole
-                                ids, buckets of 4 slots; 0 = 32) or 16 (tags, buckets of 8: id x is
+    int32_t visited_bits;     /* slot width of the visited cache of one query per warp: 0 (the library's
+                                choice: 16 when hash_slots is 0 too, the primaries are LVQ records, n
+                                allows it and a query may expand more than about 128 nodes -- 176 with
+                                LVQ-4 -- counted as max_hops, or 9/8 L without a limit; else 32), 32
+                                (whole ids, buckets of 4 slots) or 16 (tags, buckets of 8: id x is
                                 kept as x >> b in bucket (x xor (x >> b)) mod 2^b of the 2^b =
                                 slots / 8 buckets, which names x exactly; needs n <= 65535 * slots
                                 / 8, else LV_ERR_ARG; with hash_slots 0 the default slot count is

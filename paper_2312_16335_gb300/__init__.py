@@ -373,8 +373,9 @@ class Index:
         width: beam members expanded per round (1 = classic best-first).
         warps_per_query: warps sharing one query (1, 2, 4; divides width; 0 = 1);
         queries_per_warp: 1, or 2 (one query per 16 lanes; LVQ primaries, width <= 2,
-        width * R <= 128), 0 = 1.  visited_bits: slot width of the visited cache, 32 (ids; 0 =
-        32) or 16 (tags, twice the default slots in the same bytes; n <= 65535 * slots / 8).  The
+        width * R <= 128), 0 = 1.  visited_bits: slot width of the visited cache, 32 (ids),
+        16 (tags, twice the default slots in the same bytes; n <= 65535 * slots / 8) or 0 (16 for
+        long walks over LVQ records, else 32).  The
         results depend on none of these."""
         Q = _f32(Q)
         m = Q.shape[0]

@@ -125,6 +125,23 @@ int search_shape(const lv_index *idx, const lv_search_params *params, BeamParams
         p.vbits = 16;
         hs = hs16;
     }
+    // Default (no width, no slot count given) for long walks over LVQ records: 2048 tags in the 4 KB of
+    // 1024 ids.  They forget fewer ids, which pays for their slower lookup once a walk expands more than
+    // about 128 nodes (LVQ-4, whose records are cheaper to score again: 176).  20,000 queries, time with
+    // 2048 tags over 1024 ids: L = 64 / 128 / 192 / 256 without a budget 0.99 / 0.98 / 0.97 / 0.96
+    // (1M x 200, d = 64), 0.99 / 0.96 / 0.94 / 0.95 (L2, 200k x 960, d = 160), 1.00 / 1.00 / 0.99 / 0.99
+    // (LVQ-4, 300k x 768); with 64 expansions 1.00 - 1.02.  Above L = 256 the 2048 ids of the formula
+    // above would leave 16 warps on an SM instead of 24 (L = 300: 6.79 ms, 2048 tags 5.27 ms), and
+    // above about L = 330 so would 2048 tags (L = 400: 8.84 ms, 1024 tags 7.28 ms; L = 512: 11.1 and
+    // 9.0 ms, ids 19.2 ms).
+    const int walk = u.max_hops > 0 ? std::min(u.max_hops, u.L + u.L / 8) : u.L + u.L / 8;
+    bool fit24 = false;  // shrink the tags until 24 warps fit an SM
+    if (vb == 0 && params->hash_slots <= 0 && params->queries_per_warp != 2 && idx->pbits != 32 &&
+        walk > (idx->pbits == 4 ? 176 : 128) && tags_fit(idx->n, 2048)) {
+        p.vbits = 16;
+        hs = 2048;
+        fit24 = u.L > 256 && tags_fit(idx->n, 1024);
+    }
     p.Hcap = hs;
     p.hbits = 0;
     while ((1 << p.hbits) < hs) p.hbits++;
@@ -154,6 +171,11 @@ int search_shape(const lv_index *idx, const lv_search_params *params, BeamParams
     } else {
         p.Rcap = beam_rcap(p.W, p.T, idx->R);
         p.warp_smem = beam_warp_smem(p.Lcap, p.Hcap, p.vbits, p.Rcap, qbytes);
+        if (fit24 && 3 * ((size_t)(8 / p.T) * p.warp_smem + 1024) > 228 * 1024) {
+            p.Hcap = 1024;
+            p.hbits--;
+            p.warp_smem = beam_warp_smem(p.Lcap, p.Hcap, p.vbits, p.Rcap, qbytes);
+        }
         if (warps <= 0) warps = 8;
         if (warps % p.T) return fail(LV_ERR_ARG, w + ": warps_per_block must be a multiple of warps_per_query");
         while (warps > p.T && (size_t)(warps / p.T) * p.warp_smem > 227 * 1024) warps >>= 1;
