@@ -133,6 +133,16 @@ __device__ __forceinline__ int dp4a_uu(uint32_t a, uint32_t b, int c) {
     return d;
 }
 
+// The constants chunk (chunk CH) of a record whose chunks are spread over 4 lanes, as its lane
+// CH mod 4 holds it.  NC = ceil((CH + 1) / 4) chunks per lane put it last; with L2, where a norm
+// chunk follows and NC = ceil((CH + 2) / 4), it is the one before last when CH mod 4 = 3 (the norm
+// chunk, of lane (CH + 1) mod 4, is always last).
+template <int NC, bool L2>
+__device__ __forceinline__ uint4 const_chunk(const uint4 (&v)[NC], int CH) {
+    if constexpr (L2 && NC > 1) return (CH & 3) == 3 ? v[NC - 2] : v[NC - 1];
+    return v[NC - 1];
+}
+
 // L2: the score is 2 x (decoded inner product) - ||x||^2, the norm read from the record's second
 // constants chunk (chunk CH + 1)
 template <int NC, int BITS, bool L2 = false>
@@ -210,7 +220,6 @@ struct LvqIntScorer {
     template <int P>
     __device__ __forceinline__ void pass(const int *ids, float *out, int b, int cnt, int lane) const {
         const int g = lane & 3, grp = lane >> 2;
-        const int holder = (lane & ~3) | (CH & 3);
         uint4 v[P][NC];
         int j[P];
 #pragma unroll
@@ -267,22 +276,17 @@ struct LvqIntScorer {
         for (int r = 0; r < P; ++r) {
             // partial sums of one lane are < 2^24 in magnitude: exact conversions
             float s = fmaf((float)sh[r], 65536.0f, fmaf((float)sm[r], 256.0f, (float)sl[r]));
-            float dl = 0.f, lo = 0.f, x2 = 0.f;
-#pragma unroll
-            for (int t = 0; t < NC; ++t) {
-                if (g + 4 * t == CH) {
-                    dl = __uint_as_float(v[r][t].x);
-                    lo = __uint_as_float(v[r][t].y);
-                }
-                if (L2 && g + 4 * t == CH + 1) x2 = __uint_as_float(v[r][t].y);
-            }
             s += __shfl_xor_sync(FULL, s, 1);
             s += __shfl_xor_sync(FULL, s, 2);
-            dl = __shfl_sync(FULL, dl, holder);
-            lo = __shfl_sync(FULL, lo, holder);
-            float sc = fmaf(dl * scale, s, fmaf(lo, sq, cq));
-            if (L2) sc = fmaf(2.0f, sc, -__shfl_sync(FULL, x2, (lane & ~3) | ((CH + 1) & 3)));
-            if (g == 0 && j[r] < cnt) out[j[r]] = sc;
+            // every lane of the group has the sum: the one that loaded the constants chunk forms the
+            // score (the others compute with code bytes in their place and write nothing)
+            const uint4 k = const_chunk<NC, L2>(v[r], CH);
+            float sc = fmaf(__uint_as_float(k.x) * scale, s, fmaf(__uint_as_float(k.y), sq, cq));
+            if (L2) {
+                const float x2 = __shfl_sync(FULL, __uint_as_float(v[r][NC - 1].y), (lane & ~3) | ((CH + 1) & 3));
+                sc = fmaf(2.0f, sc, -x2);
+            }
+            if (g == (CH & 3) && j[r] < cnt) out[j[r]] = sc;
         }
     }
 
@@ -355,7 +359,6 @@ struct BuildScorer {
 
     __device__ __forceinline__ void score(const int *ids, float *out, int cnt, int lane) const {
         const int g = lane & 3, grp = lane >> 2;
-        const int holder = (lane & ~3) | (CH & 3);
         for (int b = 0; b < cnt; b += 16) {
             const int j0 = b + grp, j1 = b + 8 + grp;
             const int id0 = j0 < cnt ? ids[j0] : -1;
@@ -370,43 +373,27 @@ struct BuildScorer {
                 v1[t] = (c <= CH + (L2 ? 1 : 0) && id1 >= 0) ? ldg_stream(r1 + 16 * c) : make_uint4(0, 0, 0, 0);
             }
             int P0 = 0, P1 = 0;
-            float4 k0 = make_float4(0, 0, 0, 0), k1 = make_float4(0, 0, 0, 0);
-            float n0 = 0.f, n1 = 0.f;
 #pragma unroll
             for (int t = 0; t < NC; ++t) {
                 P0 += code_dot<BITS>(v0[t], qc[t]);
                 P1 += code_dot<BITS>(v1[t], qc[t]);
-                if (L2 && g + 4 * t == CH + 1) {
-                    n0 = __uint_as_float(v0[t].x);
-                    n1 = __uint_as_float(v1[t].x);
-                }
-                if (g + 4 * t == CH) {
-                    k0 = make_float4(__uint_as_float(v0[t].x), __uint_as_float(v0[t].y), __uint_as_float(v0[t].z),
-                                     __uint_as_float(v0[t].w));
-                    k1 = make_float4(__uint_as_float(v1[t].x), __uint_as_float(v1[t].y), __uint_as_float(v1[t].z),
-                                     __uint_as_float(v1[t].w));
-                }
             }
             P0 += __shfl_xor_sync(FULL, P0, 1);
             P1 += __shfl_xor_sync(FULL, P1, 1);
             P0 += __shfl_xor_sync(FULL, P0, 2);
             P1 += __shfl_xor_sync(FULL, P1, 2);
-            k0.x = __shfl_sync(FULL, k0.x, holder);
-            k0.y = __shfl_sync(FULL, k0.y, holder);
-            k0.z = __shfl_sync(FULL, k0.z, holder);
-            k0.w = __shfl_sync(FULL, k0.w, holder);
-            k1.x = __shfl_sync(FULL, k1.x, holder);
-            k1.y = __shfl_sync(FULL, k1.y, holder);
-            k1.z = __shfl_sync(FULL, k1.z, holder);
-            k1.w = __shfl_sync(FULL, k1.w, holder);
-            float s0 = build_pair_score(mu2, fdim, qd, ql, qG, qH, k0.x, k0.y, k0.z, k0.w, P0);
-            float s1 = build_pair_score(mu2, fdim, qd, ql, qG, qH, k1.x, k1.y, k1.z, k1.w, P1);
+            // the lane that loaded the constants chunk forms the score, as in LvqIntScorer::pass
+            const uint4 k0 = const_chunk<NC, L2>(v0, CH), k1 = const_chunk<NC, L2>(v1, CH);
+            float s0 = build_pair_score(mu2, fdim, qd, ql, qG, qH, __uint_as_float(k0.x), __uint_as_float(k0.y),
+                                        __uint_as_float(k0.z), __uint_as_float(k0.w), P0);
+            float s1 = build_pair_score(mu2, fdim, qd, ql, qG, qH, __uint_as_float(k1.x), __uint_as_float(k1.y),
+                                        __uint_as_float(k1.z), __uint_as_float(k1.w), P1);
             if (L2) {
                 const int h2 = (lane & ~3) | ((CH + 1) & 3);
-                s0 = l2_from_ip(s0, qN, __shfl_sync(FULL, n0, h2));
-                s1 = l2_from_ip(s1, qN, __shfl_sync(FULL, n1, h2));
+                s0 = l2_from_ip(s0, qN, __shfl_sync(FULL, __uint_as_float(v0[NC - 1].x), h2));
+                s1 = l2_from_ip(s1, qN, __shfl_sync(FULL, __uint_as_float(v1[NC - 1].x), h2));
             }
-            if (g == 0) {
+            if (g == (CH & 3)) {
                 if (j0 < cnt) out[j0] = s0;
                 if (j1 < cnt) out[j1] = s1;
             }
@@ -449,7 +436,7 @@ struct BuildWarpScorer {
     }
 
     __device__ __forceinline__ void score(const int *ids, float *out, int cnt, int lane) const {
-        const int holder = CH & 31, tslot = CH >> 5;
+        const int tslot = CH >> 5;
         for (int b = 0; b < cnt; b += U) {
             uint4 v[U][2];
 #pragma unroll
@@ -464,21 +451,18 @@ struct BuildWarpScorer {
             }
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                // the query's chunks past CH are zero, so the constants chunk adds nothing
-                int P = code_dot<BITS>(v[u][0], qc[0]) + code_dot<BITS>(v[u][1], qc[1]);
-#pragma unroll
-                for (int o = 16; o; o >>= 1) P += __shfl_xor_sync(FULL, P, o);
+                // the query's chunks past CH are zero, so the constants chunk adds nothing; the codes'
+                // sum is an integer, so one redux replaces a butterfly of shuffles, and the lane that
+                // loaded the constants chunk forms the score
+                const int P = __reduce_add_sync(FULL, code_dot<BITS>(v[u][0], qc[0]) + code_dot<BITS>(v[u][1], qc[1]));
                 const uint4 kv = tslot == 0 ? v[u][0] : v[u][1];
-                const float kd = __shfl_sync(FULL, __uint_as_float(kv.x), holder);
-                const float kl = __shfl_sync(FULL, __uint_as_float(kv.y), holder);
-                const float kG = __shfl_sync(FULL, __uint_as_float(kv.z), holder);
-                const float kH = __shfl_sync(FULL, __uint_as_float(kv.w), holder);
-                float sc = build_pair_score(mu2, fdim, qd, ql, qG, qH, kd, kl, kG, kH, P);
+                float sc = build_pair_score(mu2, fdim, qd, ql, qG, qH, __uint_as_float(kv.x), __uint_as_float(kv.y),
+                                            __uint_as_float(kv.z), __uint_as_float(kv.w), P);
                 if (L2) {
                     const uint4 nv = ((CH + 1) >> 5) == 0 ? v[u][0] : v[u][1];
                     sc = l2_from_ip(sc, qN, __shfl_sync(FULL, __uint_as_float(nv.x), (CH + 1) & 31));
                 }
-                if (lane == 0 && b + u < cnt) out[b + u] = sc;
+                if (lane == (CH & 31) && b + u < cnt) out[b + u] = sc;
             }
         }
     }
