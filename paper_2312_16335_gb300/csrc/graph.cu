@@ -157,6 +157,24 @@ __device__ __forceinline__ float smem_pair_score(const uint8_t *ra, const uint8_
     return l2_from_ip(ip, *reinterpret_cast<const float *>(ra + cb + 16), *reinterpret_cast<const float *>(rb + cb + 16));
 }
 
+// The same score by four lanes (g = lane mod 4), each with every fourth chunk; every lane of the group
+// gets it.  All 32 lanes take part.
+template <int BITS, bool L2>
+__device__ __forceinline__ float smem_pair_score4(const uint8_t *ra, const uint8_t *rb, int g, int CH, int cb, float mu2,
+                                                  float fdim) {
+    int P = 0;
+#pragma unroll 4
+    for (int c = g; c < CH; c += 4)
+        P += code_dot<BITS>(*reinterpret_cast<const uint4 *>(ra + 16 * c), *reinterpret_cast<const uint4 *>(rb + 16 * c));
+    P += __shfl_xor_sync(FULL, P, 1);
+    P += __shfl_xor_sync(FULL, P, 2);
+    const float4 ka = *reinterpret_cast<const float4 *>(ra + cb);
+    const float4 kb = *reinterpret_cast<const float4 *>(rb + cb);
+    const float ip = build_pair_score(mu2, fdim, ka.x, ka.y, ka.z, ka.w, kb.x, kb.y, kb.z, kb.w, P);
+    if (!L2) return ip;
+    return l2_from_ip(ip, *reinterpret_cast<const float *>(ra + cb + 16), *reinterpret_cast<const float *>(rb + cb + 16));
+}
+
 struct PruneParams {
     const uint8_t *prim;
     int64_t stride;  // record stride (multiple of 32)
@@ -164,37 +182,86 @@ struct PruneParams {
     float mu2, alpha, shift;
     int metric;  // 1: L2 pair scores -||y_a - y_b||^2
     int R, PMAX;
+    int slot;  // shared bytes of a staged record (see prune_slot)
     int64_t n;
     int32_t *graph;        // n x R
     // mode 0: batch nodes
     const int32_t *nodes;  // perm + b0
-    const int32_t *beams;  // nb x Lb
+    const int32_t *beams;  // nb x Lb, best first, -1 at the end
+    const float *bscores;  // nb x Lb: the beams' build scores
     int Lb;
     int32_t *newl;         // nb x R
-    // mode 1: reverse edges
+    // mode 1: reverse edges; targets whose list and new sources number lo < .. <= hi
     const int64_t *offs;   // n + 1 exclusive scan (hi: sources, lo: touched count)
     const int32_t *srcs;
     const int32_t *touched;
     const int64_t *total;  // lo 32 bits: number of touched targets
+    int lo, hi;
     int *status;
 };
+
+// an unsigned key that orders like the score (-0 and 0 alike), and back
+__device__ __forceinline__ unsigned score_key(float s) {
+    const unsigned u = __float_as_uint(s + 0.0f);
+    return u ^ ((u >> 31) ? 0xffffffffu : 0x80000000u);
+}
+__device__ __forceinline__ float key_score(unsigned k) {
+    return __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xffffffffu));
+}
+// (score, id) in one word: the larger the better, ties by the smaller id
+__device__ __forceinline__ unsigned long long pool_key(float s, int id) {
+    return (unsigned long long)score_key(s) << 32 | (unsigned)~id;
+}
+
+// Writes the values of the block's kept threads, in thread order, to dst[base ..) while they fit below
+// cap; returns base + their number.  wcnt: one int per warp.  Every thread of the block calls it.
+template <int NT>
+__device__ __forceinline__ int block_append(bool keep, int value, int *dst, int base, int cap, int *wcnt) {
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const unsigned bal = __ballot_sync(FULL, keep);
+    __syncthreads();
+    if (lane == 0) wcnt[wid] = __popc(bal);
+    __syncthreads();
+    int pos = base + __popc(bal & ((1u << lane) - 1u)), all = 0;
+#pragma unroll
+    for (int w = 0; w < NT / 32; ++w) {
+        if (w < wid) pos += wcnt[w];
+        all += wcnt[w];
+    }
+    if (keep && pos < cap) dst[pos] = value;
+    return base + all;
+}
 
 // MODE 0: pool = beam (minus p) u old out-list of p; output to newl[t].
 // MODE 1: pool = current out-list of u + its new sources (ascending, not present);
 //         pruned only when it exceeds R; output to graph[u].
-template <int BITS, int MODE, bool L2>
-__global__ void __launch_bounds__(128) prune_kernel(const PruneParams pp) {
+// One block per node.  The pool's records are staged in shared memory by 16-byte asynchronous
+// copies; ranks put the pool in order (score desc, id asc); then the kept members are taken one by
+// one, each striking out the members of the rest that it covers.  Bound by the latency of that
+// chain (one barrier per kept member) and by the shared-memory reads of the pair scores, so nothing
+// in it is serial over the pool: lists are compacted by ballots, the beam's part of the pool comes
+// with its scores and its order from the search (only the old neighbours are scored and merged in),
+// and the members still standing are bits of ballot words in rank order, one thread per member.
+// Two passes over 200,000 nodes of 160 codes (R = 64, L_build = 128): 30.4 -> 8.8 ms (mode 0) and 18.1
+// -> 7.4 ms (mode 1) against lists walked by one thread and the whole pool ranked and rescored; over
+// 50,000 nodes of 768 codes, four lanes per record: 41.6 -> 13.3 ms and 10.4 -> 5.2 ms (a thread per
+// record: 23.1 and 5.4 ms).
+template <int BITS, int MODE, bool L2, bool LONG, int NT>
+__global__ void __launch_bounds__(NT) prune_kernel(const PruneParams pp) {
+    constexpr int POOL = MODE == 0 ? LCAP_MAX + RMAX : 4 * RMAX + 256;  // the largest PMAX
+    constexpr int E = (POOL + NT - 1) / NT;                             // pool members of a lane
+    constexpr int WORDS = E * NT / 32;
+    static_assert(WORDS <= 32, "a lane reads one word");
     extern __shared__ __align__(16) unsigned char sm[];
-    const int stride = (int)pp.stride;
-    uint8_t *recs = sm;                                              // PMAX records
-    uint8_t *prec = recs + (size_t)pp.PMAX * stride;                 // own record
-    int *pid = reinterpret_cast<int *>(prec + stride);               // PMAX ids
-    float *psc = reinterpret_cast<float *>(pid + pp.PMAX);           // PMAX scores
-    int *ord = reinterpret_cast<int *>(psc + pp.PMAX);               // PMAX order
-    int *aux = ord + pp.PMAX;                                        // PMAX scratch
-    unsigned char *dead = reinterpret_cast<unsigned char *>(aux + pp.PMAX);
-    __shared__ int s_np, s_nsel, s_nl, s_out[RMAX];
-    const int tid = threadIdx.x;
+    uint8_t *const recs = sm;                                                            // PMAX records
+    uint8_t *const prec = recs + (size_t)pp.PMAX * pp.slot;                              // own record
+    unsigned long long *const key = reinterpret_cast<unsigned long long *>(prec + pp.slot);  // PMAX keys
+    int *const pid = reinterpret_cast<int *>(key + pp.PMAX);                             // PMAX ids
+    unsigned short *const ord = reinterpret_cast<unsigned short *>(pid + pp.PMAX);       // PMAX: rank -> member
+    __shared__ int s_out[RMAX], s_wcnt[NT / 32], s_np, s_self;
+    __shared__ unsigned s_mask[2][WORDS];
+    __shared__ unsigned char s_list[NT / 32][32];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
 
     int64_t p;
     int32_t *dst;
@@ -208,138 +275,202 @@ __global__ void __launch_bounds__(128) prune_kernel(const PruneParams pp) {
     }
     const int32_t *old = pp.graph + p * pp.R;
 
-    // ---- gather the pool (ordered: first list, then additions) ----
+    // records [from, to) of the pool (to == np + 1: and p's own) in 16-byte chunks, 16 or 32 lanes a record
+    const int chunks = (pp.cb + (L2 ? 32 : 16)) / 16;
+    auto stage = [&](int from, int to, bool own) {
+        const int g = chunks <= 16 ? 16 : 32;
+        for (int r = from + tid / g; r < to + (own ? 1 : 0); r += NT / g) {
+            const uint8_t *src = pp.prim + (r < to ? (int64_t)pid[r] : p) * pp.stride;
+            const uint8_t *d = r < to ? recs + (size_t)r * pp.slot : prec;
+            for (int c = tid & (g - 1); c < chunks; c += g)
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(d + 16 * c)),
+                             "l"(src + 16 * c)
+                             : "memory");
+        }
+    };
+
+    // ---- gather the pool: members [0, n0) come sorted and scored (mode 0: the beam) ----
+    int np, n0 = 0;
     if (MODE == 0) {
         // beam members except p (distinct), then old neighbours not in the beam
         const int32_t *beam = pp.beams + (int64_t)blockIdx.x * pp.Lb;
+        const float *bsc = pp.bscores + (int64_t)blockIdx.x * pp.Lb;
         if (tid == 0) {
-            int np = 0;
-            for (int t = 0; t < pp.Lb; ++t) {
-                int u = beam[t];
-                if (u < 0) break;
-                if (u != p) pid[np++] = u;
-            }
-            s_np = np;
+            s_np = 0;
+            s_self = 0x7fffffff;
         }
         __syncthreads();
-        const int nbeam = s_np;
-        // old neighbours: flag those already in the beam (parallel), then append in order
-        for (int s = tid; s < pp.R; s += blockDim.x) {
-            int u = old[s];
-            int keep = (u >= 0 && u != p) ? 1 : 0;
-            if (keep)
-                for (int t = 0; t < nbeam; ++t)
-                    if (pid[t] == u) {
-                        keep = 0;
-                        break;
-                    }
-            aux[s] = keep ? u : -1;
+        for (int t = tid; t < pp.Lb; t += NT) {
+            const int u = beam[t];
+            if (u >= 0 && (t + 1 == pp.Lb || beam[t + 1] < 0)) s_np = t + 1;
+            if (u == p) s_self = t;
         }
         __syncthreads();
-        if (tid == 0) {
-            int np = nbeam;
-            for (int s = 0; s < pp.R; ++s)
-                if (aux[s] >= 0 && np < pp.PMAX) pid[np++] = aux[s];
-            s_np = np;
+        const int nb = s_np, self = s_self;
+        n0 = nb - (self < nb ? 1 : 0);
+        for (int t = tid; t < nb; t += NT) {
+            if (t == self) continue;
+            const int u = beam[t], o = t - (t > self ? 1 : 0);
+            pid[o] = u;
+            key[o] = pool_key(bsc[t], u);
         }
         __syncthreads();
+        if (tid == 0) s_np = n0;
+        stage(0, n0, false);
+        // four threads look for each old neighbour in the beam
+        __syncthreads();
+        for (int s0 = 0; s0 < pp.R; s0 += NT / 4) {
+            const int s = s0 + (tid >> 2);
+            const int u = s < pp.R ? old[s] : -1;
+            unsigned in = 0;
+            if (u >= 0)
+                for (int t = tid & 3; t < n0; t += 4) in |= pid[t] == u ? 1u : 0u;
+            in |= __shfl_xor_sync(FULL, in, 1);
+            in |= __shfl_xor_sync(FULL, in, 2);
+            if ((tid & 3) == 0 && u >= 0 && u != p && !in) pid[atomicAdd(&s_np, 1)] = u;
+        }
+        __syncthreads();
+        np = s_np;
+        stage(n0, np, true);
     } else {
         const int64_t o0 = pp.offs[p] >> 32, o1 = pp.offs[p + 1] >> 32;
         const int nsrc = (int)(o1 - o0);
         // current list (compacted)
-        if (tid == 0) {
-            int nl = 0;
-            for (int s = 0; s < pp.R; ++s)
-                if (old[s] >= 0) pid[nl++] = old[s];
-            s_nl = nl;
+        int nl = 0;
+        for (int s0 = 0; s0 < pp.R; s0 += NT) {
+            const int s = s0 + tid, u = s < pp.R ? old[s] : -1;
+            nl = block_append<NT>(u >= 0, u, pid, nl, pp.PMAX, s_wcnt);
         }
-        __syncthreads();
-        const int nl = s_nl;
-        // sort the sources ascending (ranks; sources are distinct) and drop present ones
+        if (nl + nsrc <= pp.lo || nl + nsrc > pp.hi) return;  // the whole block: another launch's
+        // the sources ascending (ranks; they are distinct), without those present
         if (nsrc > pp.PMAX && tid == 0) atomicOr(pp.status, ST_CAPACITY);
-        for (int t = tid; t < nsrc; t += blockDim.x) {
-            const int s = pp.srcs[o0 + t];
+        int *const tmp = reinterpret_cast<int *>(key);  // PMAX ids by rank
+        int *const src = tmp + pp.PMAX;                 // the sources, when they fit
+        const bool fit = nsrc <= pp.PMAX;
+        for (int t = tid; fit && t < nsrc; t += NT) src[t] = pp.srcs[o0 + t];
+        __syncthreads();
+        for (int t = tid; t < nsrc; t += NT) {
+            const int s = fit ? src[t] : pp.srcs[o0 + t];
             int rank = 0;
-            for (int w = 0; w < nsrc; ++w) rank += pp.srcs[o0 + w] < s ? 1 : 0;
-            int keep = s != p;
-            if (keep)
-                for (int w = 0; w < nl; ++w)
-                    if (pid[w] == s) {
-                        keep = 0;
-                        break;
-                    }
-            if (rank < pp.PMAX) ord[rank] = keep ? s : -1;
+            for (int w = 0; w < nsrc; ++w) rank += (fit ? src[w] : pp.srcs[o0 + w]) < s ? 1 : 0;
+            bool keep = s != p;
+            for (int w = 0; w < nl; ++w) keep &= pid[w] != s;
+            if (rank < pp.PMAX) tmp[rank] = keep ? s : -1;
         }
         __syncthreads();
-        if (tid == 0) {
-            int np = nl;
-            for (int t = 0; t < nsrc && t < pp.PMAX; ++t)
-                if (ord[t] >= 0) {
-                    if (np < pp.PMAX)
-                        pid[np++] = ord[t];
-                    else
-                        atomicOr(pp.status, ST_CAPACITY);
-                }
-            s_np = np;
+        np = nl;
+        for (int t0 = 0; t0 < min(nsrc, pp.PMAX); t0 += NT) {
+            const int t = t0 + tid, s = t < min(nsrc, pp.PMAX) ? tmp[t] : -1;
+            np = block_append<NT>(s >= 0, s, pid, np, pp.PMAX, s_wcnt);
         }
         __syncthreads();
-        if (s_np <= pp.R) {
-            for (int s = tid; s < pp.R; s += blockDim.x) dst[s] = s < s_np ? pid[s] : -1;
+        if (np > pp.PMAX) {
+            if (tid == 0) atomicOr(pp.status, ST_CAPACITY);
+            np = pp.PMAX;
+        }
+        if (np <= pp.R) {
+            for (int s = tid; s < pp.R; s += NT) dst[s] = s < np ? pid[s] : -1;
             return;
         }
+        stage(0, np, true);
     }
-    const int np = s_np;
 
-    // ---- stage records (16-byte chunks) ----
-    const int chunks = stride / 16;
-    for (int t = tid; t < (np + 1) * chunks; t += blockDim.x) {
-        const int r = t / chunks, c = t % chunks;
-        const int64_t id = r < np ? pid[r] : p;
-        uint8_t *dstr = r < np ? recs + (size_t)r * stride : prec;
-        *reinterpret_cast<uint4 *>(dstr + 16 * c) = *reinterpret_cast<const uint4 *>(pp.prim + id * pp.stride + 16 * c);
-    }
+    // ---- score the rest, order by (score desc, id asc) ----
+    for (int i = tid; i < np; i += NT) ord[i] = (unsigned short)i;
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
     const float fdim = (float)pp.dim;
-    for (int i = tid; i < np; i += blockDim.x) {
-        psc[i] = smem_pair_score<BITS, L2>(prec, recs + (size_t)i * stride, pp.CH, pp.cb, pp.mu2, fdim);
-        dead[i] = 0;
-    }
-    __syncthreads();
-    // ---- order by (score desc, id asc) ----
-    for (int i = tid; i < np; i += blockDim.x) {
-        const float s = psc[i];
-        const int id = pid[i];
-        int rank = 0;
-        for (int t = 0; t < np; ++t) rank += key_better(psc[t], pid[t], s, id) ? 1 : 0;
-        ord[rank] = i;
-    }
-    if (tid == 0) s_nsel = 0;
-    __syncthreads();
-    // ---- greedy selection ----
-    for (int pos = 0; pos < np; ++pos) {
-        const int i = ord[pos];
-        if (dead[i]) continue;  // uniform: dead[] only changes between barriers
-        const int nsel = s_nsel;
-        if (nsel >= pp.R) break;
-        __syncthreads();
-        if (tid == 0) {
-            s_out[nsel] = pid[i];
-            s_nsel = nsel + 1;
+    if constexpr (LONG) {
+        for (int i0 = n0; i0 < np; i0 += NT / 4) {  // whole warps
+            const int i = i0 + (tid >> 2), j = min(i, np - 1);
+            const float f = smem_pair_score4<BITS, L2>(prec, recs + (size_t)j * pp.slot, tid & 3, pp.CH, pp.cb, pp.mu2, fdim);
+            if (i < np && (tid & 3) == 0) key[i] = pool_key(f, pid[i]);
         }
-        if (nsel + 1 < pp.R) {
-            const uint8_t *ri = recs + (size_t)i * stride;
-            for (int q = pos + 1 + tid; q < np; q += blockDim.x) {
-                const int j = ord[q];
-                if (dead[j]) continue;
-                const float s = smem_pair_score<BITS, L2>(ri, recs + (size_t)j * stride, pp.CH, pp.cb, pp.mu2, fdim);
-                if (__fmul_rn(pp.alpha, s) >= __fadd_rn(psc[j], pp.shift)) dead[j] = 1;
+    } else {
+        for (int i = n0 + tid; i < np; i += NT)
+            key[i] = pool_key(smem_pair_score<BITS, L2>(prec, recs + (size_t)i * pp.slot, pp.CH, pp.cb, pp.mu2, fdim), pid[i]);
+    }
+    __syncthreads();
+    for (int i = tid; i < np; i += NT) {
+        const unsigned long long k = key[i];
+        int rank = 0;
+        if (i < n0) {
+            rank = i;
+        } else {  // sorted members ahead of it
+            int hi = n0;
+            while (rank < hi) {
+                const int mid = (rank + hi) >> 1;
+                if (key[mid] > k)
+                    rank = mid + 1;
+                else
+                    hi = mid;
             }
         }
-        __syncthreads();
+#pragma unroll 4
+        for (int t = n0; t < np; ++t) rank += key[t] > k ? 1 : 0;
+        ord[rank] = (unsigned short)i;
     }
     __syncthreads();
-    const int nsel = s_nsel;
-    for (int s = tid; s < pp.R; s += blockDim.x) dst[s] = s < nsel ? s_out[s] : -1;
+    // ---- greedy selection: word e of a warp holds the members of ranks NT e + 32 wid .. + 31 ----
+    int mine[E];         // lane's member
+    unsigned word[E];    // members of the warp still standing (the same in every lane)
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+        const int q = tid + NT * e;
+        mine[e] = q < np ? ord[q] : 0;
+        word[e] = __ballot_sync(FULL, q < np);
+    }
+    int nsel = 0, cur = 0;
+    for (int buf = 0; cur < np; buf ^= 1) {
+        const int i = ord[cur];
+        if (tid == 0) s_out[nsel] = pid[i];
+        if (++nsel >= pp.R) break;
+        const uint8_t *ri = recs + (size_t)i * pp.slot;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            if (NT * e >= np) break;
+            const int first = NT * e + 32 * wid;
+            unsigned m = word[e];  // those after the member taken
+            if (first + 31 <= cur)
+                m = 0;
+            else if (first <= cur)
+                m &= ~((2u << (cur - first)) - 1u);
+            auto covered = [&](int j, float s) {
+                return __fmul_rn(pp.alpha, s) >= __fadd_rn(key_score((unsigned)(key[j] >> 32)), pp.shift);
+            };
+            if constexpr (LONG) {  // eight members at a time, four lanes each
+                const int cnt = __popc(m);
+                if (m >> lane & 1u) s_list[wid][__popc(m & ((1u << lane) - 1u))] = (unsigned char)lane;
+                __syncwarp();
+                for (int b = 0; b < cnt; b += 8) {
+                    const int src = s_list[wid][min(b + (lane >> 2), cnt - 1)];
+                    const int j = __shfl_sync(FULL, mine[e], src);
+                    const float s = smem_pair_score4<BITS, L2>(ri, recs + (size_t)j * pp.slot, lane & 3, pp.CH, pp.cb,
+                                                               pp.mu2, fdim);
+                    m &= ~__reduce_or_sync(FULL, covered(j, s) ? 1u << src : 0u);
+                }
+                __syncwarp();  // the list is read before the next one is written
+            } else {  // a thread each
+                bool a = m >> lane & 1u;
+                if (a) {
+                    const int j = mine[e];
+                    a = !covered(j, smem_pair_score<BITS, L2>(ri, recs + (size_t)j * pp.slot, pp.CH, pp.cb, pp.mu2, fdim));
+                }
+                m = __ballot_sync(FULL, a);
+            }
+            word[e] = m;
+            if (lane == 0) s_mask[buf][e * (NT / 32) + wid] = m;
+        }
+        __syncthreads();  // the words of the other buffer are read before it is written again
+        // the next member standing: the lowest bit of the words
+        const unsigned w = lane < (np + 31) / 32 ? s_mask[buf][lane] : 0u;
+        const unsigned nz = __ballot_sync(FULL, w != 0u);
+        if (nz == 0u) break;
+        const int wi = __ffs(nz) - 1;
+        cur = 32 * wi + __ffs(__shfl_sync(FULL, w, wi)) - 1;
+    }
+    __syncthreads();
+    for (int s = tid; s < pp.R; s += NT) dst[s] = s < nsel ? s_out[s] : -1;
 }
 
 __global__ void scatter_rows_kernel(const int32_t *newl, const int32_t *nodes, int nb, int R, int32_t *graph) {
@@ -462,23 +593,37 @@ int launch_entry_argmax(const uint8_t *rec, int64_t n, int64_t stride, int code_
 }
 
 // ------------------------------------------------------------------ driver
-static int prune_smem(int PMAX, int64_t stride) { return (int)(PMAX * (stride + 17) + stride + 16); }
+// the size that decides how many reverse edges of a batch a target can take (part of the result)
+static int prune_pool_bytes(int PMAX, int64_t stride) { return (int)(PMAX * (stride + 17) + stride + 16); }
+// shared bytes of the prune kernel's arrays
+static int prune_smem(int PMAX, int slot) { return PMAX * (slot + 14) + slot; }
+// records of more code chunks than this are scored by four lanes each
+constexpr int PRUNE_LONG = 16;
+// A staged record takes its codes and constants.  Where there is room its chunks are an odd number (a
+// thread per record: the 16-byte reads of consecutive records fall on different banks; 12 chunks have
+// 4-way conflicts) or 4 mod 8 (four lanes per record: those of two consecutive records do).
+static int prune_slot(int PMAX, int chunks, int metric) {
+    const int used = chunks + 1 + metric, pad = chunks > PRUNE_LONG ? (used + 3) / 8 * 8 + 4 : used | 1;
+    return prune_smem(PMAX, 16 * pad) <= 225 * 1024 ? 16 * pad : 16 * used;
+}
+
+template <int BITS, int MODE, bool L2, bool LONG, int NT>
+static int go_prune(const PruneParams &pp, unsigned grid, cudaStream_t st) {
+    const int sm = prune_smem(pp.PMAX, pp.slot);
+    if (grid == 0) return LV_OK;
+    auto k = prune_kernel<BITS, MODE, L2, LONG, NT>;
+    LV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+    k<<<grid, NT, sm, st>>>(pp);
+    LV_CHECK_LAUNCH("prune_kernel");
+    return LV_OK;
+}
 
 template <int BITS, bool L2>
 static int launch_prune_m(const PruneParams &pp, int mode, unsigned grid, cudaStream_t st) {
-    const int sm = prune_smem(pp.PMAX, pp.stride);
-    if (grid == 0) return LV_OK;
-    if (mode == 0) {
-        auto k = prune_kernel<BITS, 0, L2>;
-        LV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
-        k<<<grid, 128, sm, st>>>(pp);
-    } else {
-        auto k = prune_kernel<BITS, 1, L2>;
-        LV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
-        k<<<grid, 128, sm, st>>>(pp);
-    }
-    LV_CHECK_LAUNCH("prune_kernel");
-    return LV_OK;
+    // long records leave room for one block of a batch node's pool on an SM: eight warps
+    if (pp.CH > PRUNE_LONG)
+        return mode == 0 ? go_prune<BITS, 0, L2, true, 256>(pp, grid, st) : go_prune<BITS, 1, L2, true, 128>(pp, grid, st);
+    return mode == 0 ? go_prune<BITS, 0, L2, false, 128>(pp, grid, st) : go_prune<BITS, 1, L2, false, 128>(pp, grid, st);
 }
 
 template <int BITS>
@@ -491,12 +636,12 @@ int build_graph_impl(lv_index *idx, int R, int Lb, float alpha, int passes, int 
     const int64_t n = idx->n;
     batch = (int)std::min<int64_t>(batch, n);
     const int PMAX = Lb + R;
-    if (prune_smem(PMAX, idx->pg.stride) > 227 * 1024) return fail(LV_ERR_CAPACITY, "build: L_build + R too large");
+    if (prune_pool_bytes(PMAX, idx->pg.stride) > 227 * 1024) return fail(LV_ERR_CAPACITY, "build: L_build + R too large");
     // reverse-edge pool: the target's list plus its new sources of one batch
     int PMAX1 = std::max(PMAX, 4 * R + 256);
     // (two prune blocks per SM for short records; long records may take most of an SM's shared memory)
     const int cap1 = idx->pg.stride > 256 ? 200 * 1024 : 120 * 1024;
-    while (PMAX1 > PMAX && prune_smem(PMAX1, idx->pg.stride) > cap1) PMAX1 -= 32;
+    while (PMAX1 > PMAX && prune_pool_bytes(PMAX1, idx->pg.stride) > cap1) PMAX1 -= 32;
     cudaFree(idx->graph);
     idx->graph = nullptr;
     idx->R = 0;
@@ -601,10 +746,12 @@ int build_graph_impl(lv_index *idx, int R, int Lb, float alpha, int passes, int 
     pp.metric = idx->metric;
     pp.R = R;
     pp.PMAX = PMAX;
+    pp.slot = prune_slot(PMAX, idx->pg.code_chunks, idx->metric);
     pp.n = n;
     pp.graph = idx->graph;
     pp.beams = bid;
     pp.Lb = Lb;
+    pp.bscores = bsc;
     pp.newl = newl;
     pp.offs = offs;
     pp.srcs = srcs;
@@ -634,9 +781,17 @@ int build_graph_impl(lv_index *idx, int R, int Lb, float alpha, int passes, int 
             scatter_pairs_kernel<<<(unsigned)((tp + 255) / 256), 256, 0, st>>>(newl, perm_d + b0, nb, R, offs, cnt, srcs);
             LV_CHECK_LAUNCH("reverse-edge kernels");
             const unsigned g1 = (unsigned)std::min<int64_t>(n, tp);
-            PruneParams pr = pp;
-            pr.PMAX = PMAX1;  // a target may receive many reverse edges in one batch
-            rc = idx->pbits == 8 ? launch_prune<8>(pr, 1, g1, st) : launch_prune<4>(pr, 1, g1, st);
+            // most targets gain a few edges: pools of up to R + 32 fit many blocks on an SM; the rest
+            // (a target may receive many reverse edges in one batch) take a second launch
+            const int small = std::min(R + 32, PMAX1);
+            for (int tier = 0; tier < (small < PMAX1 ? 2 : 1) && !rc; ++tier) {
+                PruneParams pr = pp;
+                pr.PMAX = tier ? PMAX1 : small;
+                pr.slot = prune_slot(pr.PMAX, idx->pg.code_chunks, idx->metric);
+                pr.lo = tier ? small : -1;
+                pr.hi = tier || small == PMAX1 ? 0x7fffffff : small;
+                rc = idx->pbits == 8 ? launch_prune<8>(pr, 1, g1, st) : launch_prune<4>(pr, 1, g1, st);
+            }
             if (rc) return rc;
         }
     }
