@@ -81,10 +81,10 @@ struct BeamParams {
 constexpr int WMAX = 4;
 constexpr int CMAX = 256;  // candidates of one round (W * R)
 
-// shared memory of one query: beam (8 Lcap), visited cache (Hcap slots of vbits / 8 bytes), 4
-// candidate arrays (16 Rcap), the scorer's query (qbytes, a multiple of 16), control words (64)
+// shared memory of one query: beam (8 Lcap), visited cache (Hcap slots of vbits / 8 bytes), 3
+// candidate arrays (12 Rcap), the scorer's query (qbytes, a multiple of 16), control words (64)
 inline int beam_warp_smem(int Lcap, int Hcap, int vbits, int Rcap, int qbytes) {
-    return 8 * Lcap + vbits / 8 * Hcap + 16 * Rcap + qbytes + 64;  // + 16 control words
+    return 8 * Lcap + vbits / 8 * Hcap + 12 * Rcap + qbytes + 64;  // + 16 control words
 }
 // every id below n has a 16-bit tag in a cache of hcap slots (hcap / 8 buckets of 8 tags)
 inline bool tags_fit(int64_t n, int hcap) {
@@ -625,9 +625,8 @@ __global__ void __launch_bounds__(256, 3) beam_kernel(const BeamParams p) {
     uint16_t *const tags = reinterpret_cast<uint16_t *>(hash);
     int *const cI = hash + (TAGS ? p.Hcap / 2 : p.Hcap);      // ids of one expansion, then of
     float *const cS = reinterpret_cast<float *>(cI + p.Rcap);  // the candidates that enter (in place)
-    int *const vPB = reinterpret_cast<int *>(cS + p.Rcap);     // beam members ahead of each (| rank << 16)
-    int *const sPB = vPB + p.Rcap;                             // the same in candidate-rank order
-    void *const qsm = sPB + p.Rcap;                            // the scorer's query
+    int *const vPB = reinterpret_cast<int *>(cS + p.Rcap);     // beam members ahead of each | rank << 16
+    void *const qsm = vPB + p.Rcap;                            // the scorer's query
     int *const ctl = reinterpret_cast<int *>(reinterpret_cast<unsigned char *>(qsm) + PS::QBYTES);
     // ctl: [0] query, [1] size, [2] F, [4 + w] candidates of warp w, [8 + w] records scored by warp w
     // this warp's slice of the candidate arrays (Rw entries)
@@ -677,7 +676,7 @@ __global__ void __launch_bounds__(256, 3) beam_kernel(const BeamParams p) {
             ps.score(cI, cS, 1, lane);
             __syncwarp();
             if (lane == 0) {
-                bS[0] = cS[0];
+                bS[0] = fmaxf(cS[0], -INFINITY);  // NaN (a query with NaN) ranks last: keys stay ordered
                 bI[0] = entry;
                 ctl[1] = 1;
                 ctl[2] = 0;
@@ -820,13 +819,34 @@ __global__ void __launch_bounds__(256, 3) beam_kernel(const BeamParams p) {
                     tS = bS[L - 1];
                     tI = bI[L - 1] & ~(int)EXPANDED;
                 }
+                if (full && cnt > 32) {
+                    // several chunks: drop the ids below the beam first, so that the search for places
+                    // runs over the few that are left
+                    int c2 = 0;
+                    for (int j0 = 0; j0 < cnt; j0 += 32) {
+                        const int j = j0 + lane;
+                        const float s = j < cnt ? wS[j] : 0.f;
+                        const int id = j < cnt ? wI[j] : 0;
+                        const bool keep = j < cnt && key_better(fmaxf(s, -INFINITY), id, tS, tI);
+                        const unsigned bal = __ballot_sync(FULL, keep);
+                        __syncwarp();
+                        if (keep) {
+                            const int o = c2 + __popc(bal & lt);
+                            wI[o] = id;
+                            wS[o] = s;
+                        }
+                        c2 += __popc(bal);
+                    }
+                    cnt = c2;
+                    __syncwarp();
+                }
                 for (int j0 = 0; j0 < cnt; j0 += 32) {
                     const int j = j0 + lane;
                     bool valid = false;
                     float s = 0.f;
                     int id = 0, pb = 0;
                     if (j < cnt) {
-                        s = wS[j];
+                        s = fmaxf(wS[j], -INFINITY);
                         id = wI[j];
                         valid = !full || key_better(s, id, tS, tI);
                         if (valid) {
@@ -894,11 +914,12 @@ __global__ void __launch_bounds__(256, 3) beam_kernel(const BeamParams p) {
                 }
                 __syncwarp();
                 if (cv > 0) {
-                    // rank of each candidate among the candidates; sPB[rank] = beam members ahead.  An id
-                    // can appear twice in one round when two parents share a neighbour that the visited
-                    // cache did not catch (another warp's concurrent test, or a forgotten id): its copies
-                    // have equal keys and share a rank, so the ranks add up to less than 0 + .. + cv - 1.
-                    // Only then are the copies looked for (the first one is kept) and the rest ranked again.
+                    // place of each candidate in the merged beam: the beam members ahead of it and its
+                    // rank among the candidates.  An id can appear twice in one round when two parents
+                    // share a neighbour that the visited cache did not catch (another warp's concurrent
+                    // test, or a forgotten id): its copies have equal keys and share a rank, so the ranks
+                    // add up to less than 0 + .. + cv - 1.  Only then are the copies looked for (the
+                    // first one is kept) and the rest ranked again.
                     for (;;) {
                         unsigned ranks = 0;
                         for (int j = lane; j < cv; j += 32) {
@@ -906,9 +927,7 @@ __global__ void __launch_bounds__(256, 3) beam_kernel(const BeamParams p) {
                             const int id = cI[j];
                             int rank = 0;
                             for (int u = 0; u < cv; ++u) rank += key_better(cS[u], cI[u], s, id) ? 1 : 0;
-                            const int pb = vPB[j] & 0xffff;
-                            sPB[rank] = pb;
-                            vPB[j] = pb | (rank << 16);
+                            vPB[j] = (vPB[j] & 0xffff) | rank << 16;
                             ranks += (unsigned)rank;
                         }
                         if (Wr == 1 || __reduce_add_sync(FULL, ranks) == (unsigned)(cv * (cv - 1) / 2)) break;
@@ -921,7 +940,7 @@ __global__ void __launch_bounds__(256, 3) beam_kernel(const BeamParams p) {
                             if (keep) {
                                 s = cS[j];
                                 id = cI[j];
-                                pb = vPB[j];
+                                pb = vPB[j] & 0xffff;
                                 // copies before j: kept ones (already compacted) or of this chunk
                                 for (int u = 0; u < cv2; ++u) keep &= cI[u] != id;
                                 for (int u = j0; u < j; ++u) keep &= cI[u] != id;
@@ -937,46 +956,50 @@ __global__ void __launch_bounds__(256, 3) beam_kernel(const BeamParams p) {
                             cv2 += __popc(bal);
                             __syncwarp();
                         }
-                        if (cv2 == cv) break;  // equal ranks without copies: scores that do not order (NaN)
                         cv = cv2;
                     }
                     __syncwarp();
-                    // move beam members (in place, last chunk first; a member only moves right)
-                    const int first = sPB[0];
-                    for (int base = (size - 1) & ~31; base >= (first & ~31); base -= 32) {
-                        const int i = base + lane;
+                    // Merge in place, last 32 places first: a place that no candidate takes holds the beam
+                    // member that is as many places further up as candidates come before it.
+                    auto place = [&](int j) { return j < cv ? (vPB[j] & 0xffff) + (vPB[j] >> 16) : 0x7fffffff; };
+                    const int np0 = place(lane);
+                    int first = np0;
+                    for (int j = lane + 32; j < cv; j += 32) first = min(first, place(j));
+                    first = (int)__reduce_min_sync(FULL, (unsigned)first);
+                    const int nsize = min(L, size + cv);
+                    for (int base = (nsize - 1) & ~31; base >= (first & ~31); base -= 32) {
+                        const int d = base + lane;
+                        unsigned taken = __reduce_or_sync(FULL, (unsigned)(np0 - base) < 32u ? 1u << (np0 - base) : 0u);
+                        int before = __popc(__ballot_sync(FULL, np0 < base));
+                        for (int j0 = 32; j0 < cv; j0 += 32) {
+                            const int np = place(j0 + lane);
+                            taken |= __reduce_or_sync(FULL, (unsigned)(np - base) < 32u ? 1u << (np - base) : 0u);
+                            before += __popc(__ballot_sync(FULL, np < base));
+                        }
+                        const bool move = d < nsize && d >= first && !(taken >> lane & 1u);
                         float s = 0.f;
-                        int id = 0, np = L;
-                        if (i >= first && i < size) {
+                        int id = 0;
+                        if (move) {
+                            const int i = d - before - __popc(taken & lt);
                             s = bS[i];
                             id = bI[i];
-                            int lo = 0, hi = cv;
-                            while (lo < hi) {
-                                const int mid = (lo + hi) >> 1;
-                                if (sPB[mid] <= i)
-                                    lo = mid + 1;
-                                else
-                                    hi = mid;
-                            }
-                            np = i + lo;
                         }
                         __syncwarp();
-                        if (np < L) {
-                            bS[np] = s;
-                            bI[np] = id;
+                        if (move) {
+                            bS[d] = s;
+                            bI[d] = id;
                         }
                         __syncwarp();
                     }
                     // place the candidates (unexpanded)
                     for (int j = lane; j < cv; j += 32) {
-                        const int x = vPB[j];
-                        const int np = (x & 0xffff) + (x >> 16);
+                        const int np = place(j);
                         if (np < L) {
                             bS[np] = cS[j];
                             bI[np] = cI[j];
                         }
                     }
-                    size = min(L, size + cv);
+                    size = nsize;
                     F = min(F, first);
                 }
                 if (T > 1 && lane == 0) {

@@ -15,8 +15,8 @@ pytestmark = pytest.mark.gpu
     (300, 256, 8, 16, 32, 1.0, 300, 0),    # 16 chunks: a thread per record
     (300, 272, 8, 16, 32, 1.0, 300, 0),    # 17 chunks: four lanes per record
     (260, 530, 4, 8, 20, 1.02, 100, 1),    # 17 chunks of LVQ-4
-    (1200, 12, 8, 6, 16, 1.0, 1200, 0),    # one batch: hubs take more than R + 32 sources
-    (900, 300, 8, 6, 16, 1.0, 900, 0),     # the same with long records
+    (600, 12, 8, 6, 16, 1.0, 600, 0),    # one batch: hubs take more than R + 32 sources
+    (500, 300, 8, 6, 16, 1.0, 500, 0),     # the same with long records
     (400, 20, 8, 1, 1, 1.0, 64, 0),        # single-member pools and lists
     (700, 20, 8, 128, 200, 0.9, 350, 0),   # R = 128, pools of up to 328
     (33, 40, 8, 31, 33, 1.3, 33, 1),       # everything within one word
