@@ -335,7 +335,8 @@ struct BuildScorer {
     int64_t stride;
 
     static constexpr int QBYTES = 0;
-    static constexpr bool PREFETCH = false;
+    static constexpr bool PREFETCH = true;
+    __device__ __forceinline__ int rec_bytes() const { return 16 * (CH + 1 + (L2 ? 1 : 0)); }
     __device__ __forceinline__ void setup(const BeamParams &p, int64_t qi, int lane, void *, bool) {
         CH = p.prim_chunks;
         base = p.prim;
@@ -407,7 +408,8 @@ struct BuildScorer {
 template <int BITS, bool L2 = false>
 struct BuildWarpScorer {
     static constexpr int QBYTES = 0;
-    static constexpr bool PREFETCH = false;
+    static constexpr bool PREFETCH = true;
+    __device__ __forceinline__ int rec_bytes() const { return 16 * (CH + 1 + (L2 ? 1 : 0)); }
     static constexpr int U = 4;
     uint4 qc[2];
     float qd, ql, qG, qH, qN, mu2, fdim;
