@@ -2,6 +2,8 @@
 // dataset mean) and the FP64 column mean.  One warp per vector.
 #include <cuda_fp16.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 
 namespace lv {
@@ -9,13 +11,12 @@ namespace lv {
 constexpr double FIX = 1048576.0;  // 2^20: fixed point of the mean in the build score
 
 // Column mean, deterministic (a fixed summation order that depends on n and dim only).
-// Stage 1: block (c, r) sums the rows of chunk r (CM_ROWS rows) for the 4 x 32 columns of tile
-// c, each warp a strided subset of the rows (float4 loads along the row when the rows are
-// 16-byte aligned) in compensated float32 (Knuth's TwoSum keeps each addition's rounding
+// Stage 1: block (c, r) sums the rows of chunk r (CM_ROWS rows) for the columns of tile c, each
+// warp a strided subset of the rows in compensated float32 (Knuth's TwoSum keeps each addition's rounding
 // error in a second float32: about 44 significant bits, FP64 being a slow pipe here); the
 // warps' (sum, error) pairs are combined in FP64 in order; stage 2 adds the chunks in FP64
 // in order and rounds the mean to float32.
-constexpr int CM_ROWS = 2048, CM_COLS = 128;
+constexpr int CM_ROWS = 2048;
 
 struct Comp {
     float s = 0.f, e = 0.f;
@@ -29,39 +30,53 @@ struct Comp {
     __device__ __forceinline__ double value() const { return (double)s + (double)e; }
 };
 
-template <bool VEC>
+// V columns per lane (tile of 32 V columns; V = 4 wants dim % 4 == 0 and 16-byte aligned rows).  U
+// rows' loads go out before the first is added.  A chunk is one block per tile, so a database of few
+// chunks takes V = 1, which makes four times the blocks of it (10k x 128: 58 us with V = 4 and one row in
+// flight, 28 us with V = 4, U = 8, @@ with V = 1); 1M x 768 reads at @@ TB/s with V = 4.
+template <int V>
 __global__ void __launch_bounds__(256) column_sum_kernel(const float *__restrict__ X, int64_t n, int dim,
                                                          double *__restrict__ part) {
-    __shared__ double red[8][CM_COLS];
+    constexpr int U = V == 4 ? 8 : 16;
+    __shared__ double red[8][32 * V];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int c0 = blockIdx.x * CM_COLS + 4 * lane;
+    const int c0 = blockIdx.x * 32 * V + V * lane;
     const int64_t r0 = (int64_t)blockIdx.y * CM_ROWS, r1 = min(n, r0 + CM_ROWS);
-    Comp a0, a1, a2, a3;
-    if (VEC) {
-        if (c0 < dim)
-            for (int64_t i = r0 + warp; i < r1; i += 8) {
-                const float4 v = __ldg(reinterpret_cast<const float4 *>(X + i * dim + c0));
-                a0.add(v.x);
-                a1.add(v.y);
-                a2.add(v.z);
-                a3.add(v.w);
+    Comp a[V];
+    if (c0 < dim) {
+        auto load = [&](int64_t i, float *v) {
+            if constexpr (V == 4) {
+                const float4 x = __ldg(reinterpret_cast<const float4 *>(X + i * dim + c0));
+                v[0] = x.x;
+                v[1] = x.y;
+                v[2] = x.z;
+                v[3] = x.w;
+            } else {
+                v[0] = __ldg(X + i * dim + c0);
             }
-    } else {
-        for (int64_t i = r0 + warp; i < r1; i += 8) {
-            const float *row = X + i * dim;
-            if (c0 < dim) a0.add(row[c0]);
-            if (c0 + 1 < dim) a1.add(row[c0 + 1]);
-            if (c0 + 2 < dim) a2.add(row[c0 + 2]);
-            if (c0 + 3 < dim) a3.add(row[c0 + 3]);
+        };
+        int64_t i = r0 + warp;
+        for (; i + 8 * (U - 1) < r1; i += 8 * U) {
+            float v[U][V];
+#pragma unroll
+            for (int u = 0; u < U; ++u) load(i + 8 * u, v[u]);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+#pragma unroll
+                for (int e = 0; e < V; ++e) a[e].add(v[u][e]);
+        }
+        for (; i < r1; i += 8) {
+            float v[V];
+            load(i, v);
+#pragma unroll
+            for (int e = 0; e < V; ++e) a[e].add(v[e]);
         }
     }
-    red[warp][4 * lane] = a0.value();
-    red[warp][4 * lane + 1] = a1.value();
-    red[warp][4 * lane + 2] = a2.value();
-    red[warp][4 * lane + 3] = a3.value();
+#pragma unroll
+    for (int e = 0; e < V; ++e) red[warp][V * lane + e] = a[e].value();
     __syncthreads();
-    if (threadIdx.x < CM_COLS) {
-        const int c = blockIdx.x * CM_COLS + threadIdx.x;
+    if (threadIdx.x < 32 * V) {
+        const int c = blockIdx.x * 32 * V + threadIdx.x;
         double s = 0.0;
         for (int w = 0; w < 8; ++w) s += red[w][threadIdx.x];
         if (c < dim) part[(int64_t)blockIdx.y * dim + c] = s;
@@ -73,17 +88,38 @@ __global__ void column_mean_final_kernel(const double *__restrict__ part, int ch
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= dim) return;
     double s = 0.0;
-    for (int r = 0; r < chunks; ++r) s += part[(int64_t)r * dim + c];
+    constexpr int U = 32;  // loads in flight; the additions stay in order (an FP64 add takes 64 cycles)
+    int r = 0;
+    for (; r + U <= chunks; r += U) {
+        double v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) v[u] = __ldg(part + (int64_t)(r + u) * dim + c);
+#pragma unroll
+        for (int u = 0; u < U; ++u) s += v[u];
+    }
+    for (; r < chunks; ++r) s += part[(int64_t)r * dim + c];
     mean[c] = (float)(s / (double)n);
+}
+
+// The code of a = x - lower: floor(a / delta + 0.5) clamped, in IEEE float32 (delta > 0).
+__device__ __forceinline__ uint32_t lvq_code(float a, float delta, float levels) {
+    const float f = floorf(__fadd_rn(__fdiv_rn(a, delta), 0.5f));
+    return (uint32_t)fminf(fmaxf(f, 0.0f), levels);
 }
 
 // LVQ encode with 16-byte loads (dim % 4 == 0, 16-byte aligned rows): one warp per vector, a
 // persistent grid; lane l holds the float4 chunks l, l + 32, .. (at most KMAX) of v - mean in
 // registers between the min/max pass and the code pass.  The fixed-point mean (mui = mean_i
 // 2^20, exact for |mean_i| < 8) and its sums are computed once per block in shared memory.
-// Same arithmetic as lvq_encode_kernel, so the records are bit-identical.
+//
+// The codes are those of lvq_code, without its division: with r = a (1 / delta) the quotient is known
+// to 2^-15 (two roundings of a value below 2^8), so its nearest integer is the code unless r lies
+// within 1e-4 of a half -- then, about once in 5000 entries, the division is made.  (A reciprocal that
+// is not finite, or an entry that is not, fails the comparison and takes the division too.)  With one
+// division and one rounding call per entry the divisions bound the kernel: 1M x 768 1359 us (2.8 TB/s),
+// now @@; 1M x 160 424 us, now @@.
 template <int BITS, int KMAX, int G>
-__global__ void __launch_bounds__(256) lvq_encode_vec_kernel(const float *__restrict__ V, int64_t n, int dim,
+__global__ void __launch_bounds__(256, 4) lvq_encode_vec_kernel(const float *__restrict__ V, int64_t n, int dim,
                                                              const float *__restrict__ mean, uint8_t *__restrict__ rec,
                                                              int64_t stride, int code_bytes) {
     extern __shared__ uint8_t sm_raw[];
@@ -101,7 +137,8 @@ __global__ void __launch_bounds__(256) lvq_encode_vec_kernel(const float *__rest
     for (int j = threadIdx.x; j < dim; j += blockDim.x) {
         const float mj = mean[j];
         if (!(fabsf(mj) < 8.0f)) bad = 1;
-        const long long mi = __double2ll_rn((double)mj * FIX);
+        // 2^20 is a power of two: the float32 product is exact (when |mean_j| < 8, as far as it is used)
+        const long long mi = __float2ll_rn(mj * 1048576.0f);
         smean[j] = mj;
         smi[j] = (int)mi;  // only read when every |mean_j| < 8 (then |mi| < 2^23)
         pmu += mi;
@@ -141,30 +178,36 @@ __global__ void __launch_bounds__(256) lvq_encode_vec_kernel(const float *__rest
             hi = fmaxf(hi, __shfl_xor_sync(FULL, hi, o));
         }
         const float delta = __fdiv_rn(__fsub_rn(hi, lo), levels);
+        // delta = 0 (or not a number) makes no code sure
+        const float rdelta = delta > 0.0f ? __fdiv_rn(1.0f, delta) : INFINITY;
         uint8_t *r = rec + ii * stride;
         long long msum = 0;
-        int csum = 0;
+        unsigned csum = 0;
 #pragma unroll
         for (int k = 0; k < KMAX; ++k) {
             const int c = lane + G * k;
             if (act && c < nc) {
                 const float xs[4] = {x[k].x, x[k].y, x[k].z, x[k].w};
+                const int4 mi = *reinterpret_cast<const int4 *>(smi + 4 * c);
+                const int ms[4] = {mi.x, mi.y, mi.z, mi.w};
                 uint32_t cw[4];
+                bool sure = true;
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    uint32_t q = 0;
-                    if (delta > 0.0f) {
-                        float t = __fdiv_rn(__fsub_rn(xs[e], lo), delta);
-                        float f = floorf(__fadd_rn(t, 0.5f));
-                        f = fminf(fmaxf(f, 0.0f), levels);
-                        q = (uint32_t)f;
-                    }
-                    cw[e] = q;
-                    msum += (long long)(smi[4 * c + e] * (int)q);
-                    csum += (int)q;
+                    const float a = __fsub_rn(xs[e], lo);
+                    const float z = fmaf(a, rdelta, 8388608.0f);  // 2^23 + the nearest integer
+                    sure = sure && fabsf(fmaf(a, rdelta, -(z - 8388608.0f))) < 0.4999f;
+                    cw[e] = __float_as_uint(z) & 0xffu;
                 }
+                if (!sure)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) cw[e] = delta > 0.0f ? lvq_code(__fsub_rn(xs[e], lo), delta, levels) : 0u;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) msum += (long long)ms[e] * (int)cw[e];
+                const uint32_t w4 = cw[0] | (cw[1] << 8) | (cw[2] << 16) | (cw[3] << 24);
+                csum = __dp4a(w4, 0x01010101u, csum);
                 if (BITS == 8)
-                    *reinterpret_cast<uint32_t *>(r + 4 * c) = cw[0] | (cw[1] << 8) | (cw[2] << 16) | (cw[3] << 24);
+                    *reinterpret_cast<uint32_t *>(r + 4 * c) = w4;
                 else
                     *reinterpret_cast<uint16_t *>(r + 2 * c) =
                         (uint16_t)(cw[0] | (cw[1] << 4) | (cw[2] << 8) | (cw[3] << 12));
@@ -183,7 +226,7 @@ __global__ void __launch_bounds__(256) lvq_encode_vec_kernel(const float *__rest
             float mu1 = __fmul_rn(__ll2float_rn(smu), inv);
             float mf = __fmul_rn(__ll2float_rn(msum), inv);
             float Gt = __fadd_rn(__fmul_rn(lo, mu1), __fmul_rn(delta, mf));
-            float Ht = __fmul_rn(delta, __int2float_rn(csum));
+            float Ht = __fmul_rn(delta, __int2float_rn((int)csum));
             if (!mean_ok) Gt = Ht = __int_as_float(0x7fc00000);
             *reinterpret_cast<float4 *>(r + code_bytes) = make_float4(delta, lo, Gt, Ht);
         }
@@ -306,15 +349,18 @@ int launch_column_mean(const float *X, int64_t n, int dim, float *mean, cudaStre
     if (n <= 0 || dim <= 0) return LV_OK;
     const int64_t chunks = (n + CM_ROWS - 1) / CM_ROWS;
     if (chunks >= 65536) return fail(LV_ERR_ARG, "column_mean: more than 2^27 rows");
+    int dev = 0, sms = 0;
+    LV_CUDA(cudaGetDevice(&dev));
+    LV_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     double *part = nullptr;
     int rc = tmp_alloc((void **)&part, sizeof(double) * (size_t)chunks * dim, st);
     if (rc) return rc;
-    dim3 grd((unsigned)((dim + CM_COLS - 1) / CM_COLS), (unsigned)chunks);
-    if (dim % 4 == 0 && ((uintptr_t)X & 15) == 0)
-        column_sum_kernel<true><<<grd, 256, 0, st>>>(X, n, dim, part);
+    // four columns per lane once that gives the SMs two blocks each
+    if (dim % 4 == 0 && ((uintptr_t)X & 15) == 0 && chunks * ((dim + 127) / 128) >= 2 * sms)
+        column_sum_kernel<4><<<dim3((unsigned)((dim + 127) / 128), (unsigned)chunks), 256, 0, st>>>(X, n, dim, part);
     else
-        column_sum_kernel<false><<<grd, 256, 0, st>>>(X, n, dim, part);
-    column_mean_final_kernel<<<(dim + 127) / 128, 128, 0, st>>>(part, (int)chunks, n, dim, mean);
+        column_sum_kernel<1><<<dim3((unsigned)((dim + 31) / 32), (unsigned)chunks), 256, 0, st>>>(X, n, dim, part);
+    column_mean_final_kernel<<<(dim + 31) / 32, 32, 0, st>>>(part, (int)chunks, n, dim, mean);
     cudaError_t e = cudaGetLastError();
     tmp_free(part, st);
     if (e != cudaSuccess) return cuda_fail(e, "column mean kernels");
@@ -424,15 +470,17 @@ int launch_lvq_encode(const float *V, int64_t n, int dim, const float *mean, int
             LV_CHECK_LAUNCH("lvq_encode_vec_kernel");
             return LV_OK;
         };
-        // short vectors (dim <= 256): two per warp, 16 lanes each
-        if (bits == 8) {
-            if (nc <= 64) return go(lvq_encode_vec_kernel<8, 4, 16>);
-            if (nc <= 128) return go(lvq_encode_vec_kernel<8, 4, 32>);
-            return go(lvq_encode_vec_kernel<8, 8, 32>);
-        }
-        if (nc <= 64) return go(lvq_encode_vec_kernel<4, 4, 16>);
-        if (nc <= 128) return go(lvq_encode_vec_kernel<4, 4, 32>);
-        return go(lvq_encode_vec_kernel<4, 8, 32>);
+        // short vectors (dim <= 256): two per warp, 16 lanes each; no more chunks a lane than needed
+        // (registers, and with them the warps whose loads are in flight)
+        auto pick = [&](auto b) -> int {
+            constexpr int B = decltype(b)::value;
+            if (nc <= 48) return go(lvq_encode_vec_kernel<B, 3, 16>);
+            if (nc <= 64) return go(lvq_encode_vec_kernel<B, 4, 16>);
+            if (nc <= 128) return go(lvq_encode_vec_kernel<B, 4, 32>);
+            if (nc <= 192) return go(lvq_encode_vec_kernel<B, 6, 32>);
+            return go(lvq_encode_vec_kernel<B, 8, 32>);
+        };
+        return bits == 8 ? pick(std::integral_constant<int, 8>()) : pick(std::integral_constant<int, 4>());
     }
     if (bits == 8)
         lvq_encode_kernel<8><<<(unsigned)blocks, wpb * 32, 0, st>>>(V, n, dim, mean, rec, g.stride, g.code_bytes);
