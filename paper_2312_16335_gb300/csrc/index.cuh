@@ -15,6 +15,9 @@ struct lv_index {
     float *pmean = nullptr;
     uint8_t *sec = nullptr;
     float *smean = nullptr;
+    // bytes of the LVQ / FP16 stores above where they may be written again by a store of the same size
+    // (0: free and allocate)
+    size_t prim_b = 0, pmean_b = 0, sec_b = 0, smean_b = 0;
     float mu2 = 0.f;
     int R = 0;
     int32_t *graph = nullptr;

@@ -32,8 +32,8 @@ struct Comp {
 
 // V columns per lane (tile of 32 V columns; V = 4 wants dim % 4 == 0 and 16-byte aligned rows).  U
 // rows' loads go out before the first is added.  A chunk is one block per tile, so a database of few
-// chunks takes V = 1, which makes four times the blocks of it (10k x 128: 58 us with V = 4 and one row in
-// flight, 28 us with V = 4, U = 8, @@ with V = 1); 1M x 768 reads at @@ TB/s with V = 4.
+// chunks takes V = 1, which makes four times the blocks of it (10k x 128: 69 us with V = 4 and one row in
+// flight, 28 us with V = 4, U = 8, 13 us with V = 1); 1M x 768 reads at 6.9 TB/s with V = 4 (6.1 before).
 template <int V>
 __global__ void __launch_bounds__(256) column_sum_kernel(const float *__restrict__ X, int64_t n, int dim,
                                                          double *__restrict__ part) {
@@ -83,22 +83,34 @@ __global__ void __launch_bounds__(256) column_sum_kernel(const float *__restrict
     }
 }
 
-__global__ void column_mean_final_kernel(const double *__restrict__ part, int chunks, int64_t n, int dim,
-                                         float *__restrict__ mean) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= dim) return;
+// Stage 2: one block per 32 columns.  The chunks are added in order by one warp (an FP64 add takes 64
+// cycles here), from tiles that the other warps bring into shared memory meanwhile (489 chunks of 768
+// columns: 44 us when the adding thread loads them itself, 22 us so).
+constexpr int CF_TILE = 56;  // chunks of a tile: 8 for each of the seven loading warps
+__global__ void __launch_bounds__(256) column_mean_final_kernel(const double *__restrict__ part, int chunks, int64_t n,
+                                                                int dim, float *__restrict__ mean) {
+    __shared__ double tile[2][CF_TILE][32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = blockIdx.x * 32 + lane;
+    auto fetch = [&](int r0, int buf) {  // warps 1 .. 7
+        if (warp == 0) return;
+#pragma unroll
+        for (int u = 0; u < CF_TILE / 7; ++u) {
+            const int k = (warp - 1) + 7 * u;
+            if (r0 + k < chunks && c < dim) tile[buf][k][lane] = __ldg(part + (int64_t)(r0 + k) * dim + c);
+        }
+    };
+    fetch(0, 0);
+    __syncthreads();
     double s = 0.0;
-    constexpr int U = 32;  // loads in flight; the additions stay in order (an FP64 add takes 64 cycles)
-    int r = 0;
-    for (; r + U <= chunks; r += U) {
-        double v[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) v[u] = __ldg(part + (int64_t)(r + u) * dim + c);
-#pragma unroll
-        for (int u = 0; u < U; ++u) s += v[u];
+    for (int r0 = 0, buf = 0; r0 < chunks; r0 += CF_TILE, buf ^= 1) {
+        fetch(r0 + CF_TILE, buf ^ 1);
+        if (warp == 0) {
+            const int m = min(CF_TILE, chunks - r0);
+            for (int k = 0; k < m; ++k) s += tile[buf][k][lane];
+        }
+        __syncthreads();
     }
-    for (; r < chunks; ++r) s += part[(int64_t)r * dim + c];
-    mean[c] = (float)(s / (double)n);
+    if (warp == 0 && c < dim) mean[c] = (float)(s / (double)n);
 }
 
 // The code of a = x - lower: floor(a / delta + 0.5) clamped, in IEEE float32 (delta > 0).
@@ -117,7 +129,7 @@ __device__ __forceinline__ uint32_t lvq_code(float a, float delta, float levels)
 // within 1e-4 of a half -- then, about once in 5000 entries, the division is made.  (A reciprocal that
 // is not finite, or an entry that is not, fails the comparison and takes the division too.)  With one
 // division and one rounding call per entry the divisions bound the kernel: 1M x 768 1359 us (2.8 TB/s),
-// now @@; 1M x 160 424 us, now @@.
+// now 690 us (5.6 TB/s); 1M x 160 424 us, now 238 us.
 template <int BITS, int KMAX, int G>
 __global__ void __launch_bounds__(256, 4) lvq_encode_vec_kernel(const float *__restrict__ V, int64_t n, int dim,
                                                              const float *__restrict__ mean, uint8_t *__restrict__ rec,
@@ -360,7 +372,7 @@ int launch_column_mean(const float *X, int64_t n, int dim, float *mean, cudaStre
         column_sum_kernel<4><<<dim3((unsigned)((dim + 127) / 128), (unsigned)chunks), 256, 0, st>>>(X, n, dim, part);
     else
         column_sum_kernel<1><<<dim3((unsigned)((dim + 31) / 32), (unsigned)chunks), 256, 0, st>>>(X, n, dim, part);
-    column_mean_final_kernel<<<(dim + 31) / 32, 32, 0, st>>>(part, (int)chunks, n, dim, mean);
+    column_mean_final_kernel<<<(dim + 31) / 32, 256, 0, st>>>(part, (int)chunks, n, dim, mean);
     cudaError_t e = cudaGetLastError();
     tmp_free(part, st);
     if (e != cudaSuccess) return cuda_fail(e, "column mean kernels");
