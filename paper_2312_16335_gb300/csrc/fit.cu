@@ -277,6 +277,279 @@ __global__ void f64_to_f32_kernel(const double *__restrict__ a, int64_t n, float
     if (t < n) b[t] = (float)a[t];
 }
 
+// ------------------------------------------------- Jacobi eigh of small matrices
+// The whole decomposition of a matrix of up to JC_MAX rows in one launch: a cluster of JC_CL blocks
+// keeps A in its shared memory (row i in block i mod JC_CL, entries j >= i; two copies, one read and
+// one written in turn) and goes from round to round over the cluster barrier.  A round on the
+// pairs (p_k, q_k) splits A into 2 x 2 blocks (pair I x pair J), each owned by one thread, which reads it
+// from the old copy, applies both rotations and writes it to the new one; every block forms all
+// rotations itself.  The rotations are kept, and jacobi_vectors_kernel applies them to the rows of V,
+// which do not depend on one another, over all SMs.
+//
+// FP64 bounds this: the pipe takes a warp instruction every 64 cycles, so a division or a root
+// costs 550 and no extra warp hides it.  Hence the angle comes from float32 (any t serves that
+// brings a_pq down -- 1e-7 of it remains, the next sweep's share), and only c = 1 / sqrt(1 + t^2) and
+// s = t c are made accurate to FP64: a float32 rsqrt with one cubic step.  The update multiplies by t
+// and scales by c_I c_J at the end (12 instead of 16 operations).
+// 128 rows, 7 sweeps of 127 rounds: 5.4 ms of kernels and 2 ms of graph building with two launches a
+// round replayed from a graph made per call, 2.7 ms and 0.2 ms for the vectors now.
+constexpr int JC_CL = 16, JC_MAX = 256, JC_SWEEPS = 40;
+
+__device__ __forceinline__ double ld_cluster(uint32_t addr, int rank) {
+    uint32_t ra;
+    double v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(addr), "r"(rank));
+    asm volatile("ld.shared::cluster.f64 %0, [%1];" : "=d"(v) : "r"(ra) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_cluster(uint32_t addr, int rank, double v) {
+    uint32_t ra;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(addr), "r"(rank));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(ra), "d"(v) : "memory");
+}
+__device__ __forceinline__ void cluster_barrier() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// tangent t and cosine c of the rotation that (nearly) zeroes a_pq: rows p <- c (p - t q), q <- c (q + t p)
+__device__ __forceinline__ void jacobi_angle(double app, double aqq, double apq, double &t, double &c) {
+    t = 0.0;
+    c = 1.0;
+    if (!(fabs(apq) > 1e-300)) return;
+    const double d = aqq - app, x2 = apq + apq;
+    // scaled by a power of two to fit float32
+    const int ed = __double2hiint(d) & 0x7ff00000, ex = __double2hiint(x2) & 0x7ff00000;
+    const int e = min(max(max(ed, ex), 0x00100000), 0x7fd00000);
+    const double sc = __hiloint2double(0x7fe00000 - e, 0);
+    const float theta = __double2float_rn(d * sc) / __double2float_rn(x2 * sc);
+    const float tf = copysignf(1.0f / (fabsf(theta) + sqrtf(fmaf(theta, theta, 1.0f))), theta);
+    if (!(fabsf(tf) <= 1.0f)) return;  // 0 / 0
+    t = (double)tf;
+    const double u = fma(t, t, 1.0);
+    const double y = (double)rsqrtf(fmaf(tf, tf, 1.0f));
+    const double r = fma(-u, y * y, 1.0);  // about 2^-23: y (1 + r / 2 + 3 r^2 / 8) is good to r^3
+    c = fma(y * r, fma(0.375, r, 0.5), y);
+}
+
+// pair k of round r on Dp (even) indices, as rr_pair, with 0 <= r < Dp - 1
+__device__ __forceinline__ void rr_pair_fast(int r, int k, int Dp, int &p, int &q) {
+    const int m = Dp - 1;
+    int a = r + k, b = r - k;
+    if (a >= m) a -= m;
+    if (b < 0) b += m;
+    if (k == 0) {
+        a = r;
+        b = m;
+    }
+    p = min(a, b);
+    q = max(a, b);
+}
+
+// T threads; NB: 2 x 2 blocks of a thread at most
+template <int T, int NB>
+__global__ void __launch_bounds__(T) jacobi_cluster_kernel(double *__restrict__ A, int Dp, double2 *__restrict__ rot,
+                                                           int *__restrict__ sweeps) {
+    extern __shared__ double sm_a[];
+    __shared__ double2 s_tc[JC_MAX / 2];
+    __shared__ double s_red[T / 32][2], s_part[2];
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    uint32_t crank;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
+    const int rank = (int)crank, h = Dp / 2, rows = (Dp + JC_CL - 1) / JC_CL, rounds = Dp - 1;
+    const uint32_t base = (uint32_t)__cvta_generic_to_shared(sm_a);
+    const uint32_t part = (uint32_t)__cvta_generic_to_shared(s_part);
+    auto at = [&](int buf, int i, int j) {  // i <= j
+        return base + 8u * (uint32_t)((buf * rows + (i >> 4)) * Dp + j);
+    };
+    static_assert(JC_CL == 16, "row to block by shifts");
+    for (int l = wid; l < rows; l += T / 32) {
+        const int i = rank + JC_CL * l;
+        if (i < Dp)
+            for (int j = i + lane; j < Dp; j += 32) sm_a[l * Dp + j] = A[(int64_t)i * Dp + j];
+    }
+    // this thread's 2 x 2 blocks: pairs I < J of the round's list, the same positions in every round
+    int bI[NB], bJ[NB];
+#pragma unroll
+    for (int e = 0; e < NB; ++e) {
+        int b = (rank * T + tid) + e * JC_CL * T, i = 0;
+        if (b < h * (h - 1) / 2) {
+            while (b >= h - 1 - i) {
+                b -= h - 1 - i;
+                ++i;
+            }
+            bI[e] = i;
+            bJ[e] = i + 1 + b;
+        } else {
+            bI[e] = -1;
+            bJ[e] = 0;
+        }
+    }
+    cluster_barrier();
+    int buf = 0, sweep = 0;
+    for (;; ++sweep) {
+        // off-diagonal and diagonal sums of squares, added in one order by every block
+        double off = 0.0, diag = 0.0;
+        for (int l = wid; l < rows; l += T / 32) {
+            const int i = rank + JC_CL * l;
+            if (i < Dp)
+                for (int j = i + lane; j < Dp; j += 32) {
+                    const double v = sm_a[(buf * rows + l) * Dp + j];
+                    if (j == i)
+                        diag = fma(v, v, diag);
+                    else
+                        off = fma(v, v, off);
+                }
+        }
+        for (int o = 16; o; o >>= 1) {
+            off += __shfl_xor_sync(FULL, off, o);
+            diag += __shfl_xor_sync(FULL, diag, o);
+        }
+        if (lane == 0) {
+            s_red[wid][0] = off;
+            s_red[wid][1] = diag;
+        }
+        __syncthreads();
+        if (tid < 2) {
+            double v = 0.0;
+            for (int w = 0; w < T / 32; ++w) v += s_red[w][tid];
+            s_part[tid] = v;
+        }
+        cluster_barrier();
+        off = diag = 0.0;
+        for (int c = 0; c < JC_CL; ++c) {
+            off += ld_cluster(part, c);
+            diag += ld_cluster(part + 8, c);
+        }
+        off *= 2.0;
+        const double tot = off + diag;
+        if (!(off > 1e-28 * tot) || tot == 0.0 || sweep == JC_SWEEPS) break;
+        for (int r = 0; r < rounds; ++r, buf ^= 1) {
+            double app = 0.0, aqq = 0.0, apq = 0.0;
+            int p = 0, q = 0;
+            if (tid < h) {
+                rr_pair_fast(r, tid, Dp, p, q);
+                app = ld_cluster(at(buf, p, p), p & 15);
+                aqq = ld_cluster(at(buf, q, q), q & 15);
+                apq = ld_cluster(at(buf, p, q), p & 15);
+            }
+            // entries (p_I, p_J), (p_I, q_J), (q_I, p_J), (q_I, q_J)
+            double v[NB][4];
+            uint32_t ad[NB][4];
+            int rk[NB][4];
+#pragma unroll
+            for (int e = 0; e < NB; ++e) {
+                if (bI[e] < 0) continue;
+                int i2[2], j2[2];
+                rr_pair_fast(r, bI[e], Dp, i2[0], i2[1]);
+                rr_pair_fast(r, bJ[e], Dp, j2[0], j2[1]);
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    const int i = min(i2[x >> 1], j2[x & 1]), j = max(i2[x >> 1], j2[x & 1]);
+                    ad[e][x] = at(0, i, j);
+                    rk[e][x] = i & 15;
+                    v[e][x] = ld_cluster(ad[e][x] + 8u * (uint32_t)(buf * rows * Dp), rk[e][x]);
+                }
+            }
+            if (tid < h) {
+                double t, c;
+                jacobi_angle(app, aqq, apq, t, c);
+                s_tc[tid] = make_double2(t, c);
+                if ((tid & 15) == rank) {  // the pair's own 2 x 2 block
+                    const double c2 = c * c, tx = t * apq;
+                    st_cluster(at(buf ^ 1, p, p), p & 15, c2 * fma(t, fma(t, aqq, -2.0 * apq), app));
+                    st_cluster(at(buf ^ 1, q, q), q & 15, c2 * fma(t, fma(t, app, 2.0 * apq), aqq));
+                    st_cluster(at(buf ^ 1, p, q), p & 15, c2 * fma(t, (app - aqq) - tx, apq));
+                    rot[((int64_t)sweep * rounds + r) * h + tid] = make_double2(c, t * c);
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int e = 0; e < NB; ++e) {
+                if (bI[e] < 0) continue;
+                const double2 ti = s_tc[bI[e]], tj = s_tc[bJ[e]];
+                const double a = fma(-ti.x, v[e][2], v[e][0]), b = fma(-ti.x, v[e][3], v[e][1]);
+                const double c = fma(ti.x, v[e][0], v[e][2]), d = fma(ti.x, v[e][1], v[e][3]);
+                const double cc = ti.y * tj.y;
+                const uint32_t o = 8u * (uint32_t)((buf ^ 1) * rows * Dp);
+                st_cluster(ad[e][0] + o, rk[e][0], cc * fma(-tj.x, b, a));
+                st_cluster(ad[e][1] + o, rk[e][1], cc * fma(tj.x, a, b));
+                st_cluster(ad[e][2] + o, rk[e][2], cc * fma(-tj.x, d, c));
+                st_cluster(ad[e][3] + o, rk[e][3], cc * fma(tj.x, c, d));
+            }
+            cluster_barrier();
+        }
+    }
+    for (int l = tid; l < rows; l += T) {
+        const int i = rank + JC_CL * l;
+        if (i < Dp) A[(int64_t)i * Dp + i] = sm_a[(buf * rows + l) * Dp + i];
+    }
+    if (rank == 0 && tid == 0) *sweeps = sweep;
+    cluster_barrier();  // no block leaves while another may read its partial sums
+}
+
+// Row blockIdx.x of V: the unit row times all rotations in order; one thread per pair.
+__global__ void jacobi_vectors_kernel(const double2 *__restrict__ rot, const int *__restrict__ sweeps, int Dp,
+                                      double *__restrict__ V) {
+    __shared__ double v[JC_MAX];
+    const int k = threadIdx.x, h = Dp / 2;
+    v[k] = k == (int)blockIdx.x ? 1.0 : 0.0;
+    v[k + h] = k + h == (int)blockIdx.x ? 1.0 : 0.0;
+    const int64_t total = (int64_t)*sweeps * (Dp - 1);
+    double2 next = total > 0 ? rot[k] : make_double2(1.0, 0.0);
+    __syncthreads();
+    int r = 0;
+    for (int64_t g = 0; g < total; ++g) {
+        const double2 cs = next;
+        if (g + 1 < total) next = rot[(g + 1) * h + k];
+        int p, q;
+        rr_pair_fast(r, k, Dp, p, q);
+        const double a = v[p], b = v[q];
+        v[p] = fma(cs.x, a, -(cs.y * b));
+        v[q] = fma(cs.y, a, cs.x * b);
+        if (++r == Dp - 1) r = 0;
+        __syncthreads();
+    }
+    V[(int64_t)blockIdx.x * Dp + k] = v[k];
+    V[(int64_t)blockIdx.x * Dp + k + h] = v[k + h];
+}
+
+// Runs the cluster path on the padded matrix A (diagonal replaced by the eigenvalues) and writes V.
+// False when the device cannot hold the cluster (nothing launched).
+static int jacobi_cluster(double *A, double *V, int Dp, int *sweeps_dev, double2 *rot, cudaStream_t st, bool *ran) {
+    *ran = false;
+    const int rows = (Dp + JC_CL - 1) / JC_CL;
+    const size_t smem = sizeof(double) * 2 * (size_t)rows * Dp;
+    auto go = [&](auto kern, int threads) -> int {
+        LV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        LV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(JC_CL);
+        cfg.blockDim = dim3((unsigned)threads);
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = JC_CL;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg) != cudaSuccess || clusters < 1) {
+            cudaGetLastError();
+            return LV_OK;
+        }
+        LV_CUDA(cudaLaunchKernelEx(&cfg, kern, A, Dp, rot, sweeps_dev));
+        *ran = true;
+        return LV_OK;
+    };
+    // blocks of a thread: h (h - 1) / 2 of them, h = Dp / 2, over 16 T threads
+    int rc = Dp <= 128 ? go(jacobi_cluster_kernel<128, 1>, 128) : go(jacobi_cluster_kernel<256, 2>, 256);
+    if (rc || !*ran) return rc;
+    jacobi_vectors_kernel<<<Dp, Dp / 2, 0, st>>>(rot, sweeps_dev, Dp, V);
+    LV_CHECK_LAUNCH("jacobi_vectors_kernel");
+    return LV_OK;
+}
+
 bool eigh_top_ok(int D, int nout);
 int eigh_top(const double *K, int D, int nout, double *evals, double *evecs, cudaStream_t st);
 
@@ -292,7 +565,8 @@ int eigh_impl(const double *K, int D, int nout, double *evals, double *evecs, cu
     const int Dp = D + (D & 1);
     double *A = nullptr, *V = nullptr, *acc = nullptr, *dg = nullptr;
     double2 *cs = nullptr;
-    int *idx_d = nullptr;
+    double2 *rot = nullptr;
+    int *idx_d = nullptr, *nsw = nullptr;
     int rc = LV_OK;
     std::vector<double> diag(Dp);
     std::vector<int> order(Dp);
@@ -318,6 +592,23 @@ int eigh_impl(const double *K, int D, int nout, double *evals, double *evecs, cu
         goto done;
     }
     pad_copy_kernel<<<(unsigned)(((int64_t)Dp * Dp + 255) / 256), 256, 0, st>>>(K, D, A, V, Dp);
+    if (Dp <= JC_MAX) {
+        bool ran = false;
+        const size_t rots = (size_t)JC_SWEEPS * (Dp - 1) * (Dp / 2);
+        if (tmp_alloc((void **)&rot, sizeof(double2) * rots, st) || tmp_alloc((void **)&nsw, sizeof(int), st)) {
+            rc = fail(LV_ERR_OOM, "eigh: allocation failed");
+            goto done;
+        }
+        if ((rc = jacobi_cluster(A, V, Dp, nsw, rot, st, &ran))) goto done;
+        if (ran) {
+            if (sweeps_out && (cudaMemcpyAsync(&sweep, nsw, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+                               cudaStreamSynchronize(st) != cudaSuccess)) {
+                rc = fail(LV_ERR_CUDA, "eigh: kernel failure");
+                goto done;
+            }
+            goto sorted;
+        }
+    }
     // one sweep = Dp - 1 rounds of (rotation angles, fused round); captured once into a CUDA
     // graph (launched per sweep), else launched directly
     if (fused && Dp * 32 > 48 * 1024 &&
@@ -363,6 +654,7 @@ int eigh_impl(const double *K, int D, int nout, double *evals, double *evecs, cu
             goto done;
         }
     }
+sorted:
     // sort eigenvalues descending (stable by index); the padding index (D) is dropped
     {
         diag_kernel<<<(Dp + 255) / 256, 256, 0, st>>>(A, Dp, dg);
@@ -392,6 +684,8 @@ done:
     tmp_free(cs, st);
     tmp_free(idx_d, st);
     tmp_free(dg, st);
+    tmp_free(rot, st);
+    tmp_free(nsw, st);
     return rc;
 }
 

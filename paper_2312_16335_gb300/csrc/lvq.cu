@@ -155,8 +155,12 @@ __global__ void __launch_bounds__(256, 4) lvq_encode_vec_kernel(const float *__r
         smi[j] = (int)mi;  // only read when every |mean_j| < 8 (then |mi| < 2^23)
         pmu += mi;
     }
-    atomicAdd(reinterpret_cast<unsigned long long *>(&s_mu), (unsigned long long)pmu);
-    if (bad) atomicOr(&s_bad, 1);
+    for (int o = 16; o; o >>= 1) pmu += __shfl_xor_sync(FULL, pmu, o);
+    bad = __any_sync(FULL, bad);
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(reinterpret_cast<unsigned long long *>(&s_mu), (unsigned long long)pmu);
+        if (bad) atomicOr(&s_bad, 1);
+    }
     __syncthreads();
     const bool mean_ok = !s_bad;
     const long long smu = s_mu;

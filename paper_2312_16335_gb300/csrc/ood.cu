@@ -80,6 +80,45 @@ static int gemm_small(int M, int N, int K, T alpha, const T *A, int lda, bool ta
     return LV_OK;
 }
 
+// C (M x N) = op(A) op(B) in FP64.  One output per thread, 8 x 8 outputs a block: a warp gets an FP64
+// instruction through every 64 cycles whatever else runs, so the d x d and d x D products of the
+// polar factor spread over all schedulers of the chip instead of 4 blocks of 64 x 64 outputs
+// (128 x 128 x 512: 350 us, 44 us now).
+__global__ void __launch_bounds__(64) gemm_f64_kernel(int M, int N, int K, const double *__restrict__ A, int lda, bool ta,
+                                                      const double *__restrict__ B, int ldb, bool tb,
+                                                      double *__restrict__ C, int ldc) {
+    __shared__ double As[32][9], Bs[32][9];
+    const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3, r0 = blockIdx.y * 8, c0 = blockIdx.x * 8;
+    double acc = 0.0;
+    for (int k0 = 0; k0 < K; k0 += 32) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int t = threadIdx.x + 64 * u;
+            // along the operand's rows: k of a plain A or a transposed B, else the tile's side
+            const int ka = ta ? t >> 3 : t & 31, i = ta ? t & 7 : t >> 5;
+            As[ka][i] = (r0 + i < M && k0 + ka < K)
+                            ? (ta ? A[(int64_t)(k0 + ka) * lda + r0 + i] : A[(int64_t)(r0 + i) * lda + k0 + ka])
+                            : 0.0;
+            const int kb = tb ? t & 31 : t >> 3, j = tb ? t >> 5 : t & 7;
+            Bs[kb][j] = (c0 + j < N && k0 + kb < K)
+                            ? (tb ? B[(int64_t)(c0 + j) * ldb + k0 + kb] : B[(int64_t)(k0 + kb) * ldb + c0 + j])
+                            : 0.0;
+        }
+        __syncthreads();
+#pragma unroll 8
+        for (int k = 0; k < 32; ++k) acc = fma(As[k][ty], Bs[k][tx], acc);
+        __syncthreads();
+    }
+    if (r0 + ty < M && c0 + tx < N) C[(int64_t)(r0 + ty) * ldc + c0 + tx] = acc;
+}
+
+static int gemm_f64(int M, int N, int K, const double *A, int lda, bool ta, const double *B, int ldb, bool tb, double *C,
+                    int ldc, cudaStream_t st) {
+    gemm_f64_kernel<<<dim3((N + 7) / 8, (M + 7) / 8), 64, 0, st>>>(M, N, K, A, lda, ta, B, ldb, tb, C, ldc);
+    LV_CHECK_LAUNCH("gemm_f64_kernel");
+    return LV_OK;
+}
+
 // out[slot] += <X, Y>_F (sum of elementwise products), FP64 accumulation of float32 data
 __global__ void frob_dot_kernel(const float *__restrict__ X, const float *__restrict__ Y, int64_t n, double *out) {
     __shared__ double sh[256];
@@ -136,19 +175,22 @@ __global__ void f64_to_f32_k(const double *__restrict__ a, int64_t n, float *__r
     if (t < n) b[t] = (float)a[t];
 }
 
-// W = U diag(w) U^T with w_i = 1/sqrt(lambda_i) (0 for lambda_i <= 1e-12 lambda_max); U rows = eigvecs
-__global__ void inv_sqrt_kernel(const double *__restrict__ evals, const double *__restrict__ U, int d,
-                                double *__restrict__ W) {
-    const int i = blockIdx.y, j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= d) return;
-    const double lmax = evals[0];
-    double s = 0.0;
-    for (int r = 0; r < d; ++r) {
+// Us = diag(w) U for the rows (eigenvectors) of U (d x d).  CLIP: w = 1 / sqrt(lambda) above 1, else 1;
+// otherwise w = 1 / sqrt(lambda), 0 for lambda <= 1e-12 lambda_max.  One block per row.
+template <bool CLIP>
+__global__ void scale_rows_kernel(const double *__restrict__ evals, const double *__restrict__ U, int d,
+                                  double *__restrict__ Us) {
+    __shared__ double w;
+    const int64_t r = blockIdx.x;
+    if (threadIdx.x == 0) {
         const double l = evals[r];
-        const double w = (l > 1e-12 * lmax && l > 0.0) ? 1.0 / sqrt(l) : 0.0;
-        s += U[(int64_t)r * d + i] * w * U[(int64_t)r * d + j];
+        if (CLIP)
+            w = l > 1.0 ? 1.0 / sqrt(l) : 1.0;
+        else
+            w = (l > 1e-12 * evals[0] && l > 0.0) ? 1.0 / sqrt(l) : 0.0;
     }
-    W[(int64_t)i * d + j] = s;
+    __syncthreads();
+    for (int j = threadIdx.x; j < d; j += blockDim.x) Us[r * d + j] = w * U[r * d + j];
 }
 
 // ---------------------------------------------------------------- context
@@ -219,14 +261,14 @@ static int polar_dev(OodCtx &c, const float *C, float *S) {
     const int64_t nd = (int64_t)d * D;
     f32_to_f64_k<<<(unsigned)((nd + 255) / 256), 256, 0, c.st>>>(C, nd, c.C64);
     LV_CHECK_LAUNCH("f32_to_f64_k");
-    int rc = gemm_small<double>(d, d, D, 1.0, c.C64, D, false, c.C64, D, true, 0.0, c.G64, d, c.st);
+    int rc = gemm_f64(d, d, D, c.C64, D, false, c.C64, D, true, c.G64, d, c.st);
     if (rc) return rc;
     rc = eigh_impl(c.G64, d, d, c.ev64, c.U64, c.st, nullptr);
     if (rc) return rc;
-    inv_sqrt_kernel<<<dim3((d + 127) / 128, d), 128, 0, c.st>>>(c.ev64, c.U64, d, c.W64);
-    LV_CHECK_LAUNCH("inv_sqrt_kernel");
-    rc = gemm_small<double>(d, D, d, 1.0, c.W64, d, false, c.C64, D, false, 0.0, c.S64, D, c.st);
-    if (rc) return rc;
+    scale_rows_kernel<false><<<d, 128, 0, c.st>>>(c.ev64, c.U64, d, c.S64);
+    LV_CHECK_LAUNCH("scale_rows_kernel");
+    if ((rc = gemm_f64(d, d, d, c.U64, d, true, c.S64, d, false, c.W64, d, c.st))) return rc;
+    if ((rc = gemm_f64(d, D, d, c.W64, d, false, c.C64, D, false, c.S64, D, c.st))) return rc;
     f64_to_f32_k<<<(unsigned)((nd + 255) / 256), 256, 0, c.st>>>(c.S64, nd, S);
     LV_CHECK_LAUNCH("f64_to_f32_k");
     return LV_OK;
@@ -316,20 +358,6 @@ static int brent_min(F &&func, double a, double b, double xatol, int maxit, doub
     return LV_OK;
 }
 
-// W = U diag(min(1, 1/sigma_i)) U^T with sigma_i^2 the eigenvalues of A A^T
-__global__ void clip_scale_kernel(const double *__restrict__ evals, const double *__restrict__ U, int d,
-                                  double *__restrict__ W) {
-    const int i = blockIdx.y, j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= d) return;
-    double s = 0.0;
-    for (int r = 0; r < d; ++r) {
-        const double l = evals[r];
-        const double w = l > 1.0 ? 1.0 / sqrt(l) : 1.0;
-        s += U[(int64_t)r * d + i] * w * U[(int64_t)r * d + j];
-    }
-    W[(int64_t)i * d + j] = s;
-}
-
 }  // namespace lv
 
 using namespace lv;
@@ -348,7 +376,7 @@ int leanvec_spectral_clip(float *A, int d, int D, lv_stream_t stream) {
         rc = fail(LV_ERR_OOM, "spectral_clip: allocation failed");
     if (rc == LV_OK) {
         f32_to_f64_k<<<(unsigned)((dD + 255) / 256), 256, 0, st>>>(A, (int64_t)dD, A64);
-        rc = gemm_small<double>(d, d, D, 1.0, A64, D, false, A64, D, true, 0.0, G, d, st);
+        rc = gemm_f64(d, d, D, A64, D, false, A64, D, true, G, d, st);
     }
     if (rc == LV_OK) rc = d > 1 ? eigh_impl(G, d, d, ev, U, st, nullptr) : LV_OK;
     if (rc == LV_OK && d == 1) {
@@ -358,8 +386,10 @@ int leanvec_spectral_clip(float *A, int d, int D, lv_stream_t stream) {
         cudaMemcpyAsync(U, &one, 8, cudaMemcpyHostToDevice, st);
     }
     if (rc == LV_OK) {
-        clip_scale_kernel<<<dim3((d + 127) / 128, d), 128, 0, st>>>(ev, U, d, W);
-        rc = gemm_small<double>(d, D, d, 1.0, W, d, false, A64, D, false, 0.0, R, D, st);
+        // A <- U^T diag(w) U A
+        scale_rows_kernel<true><<<d, 128, 0, st>>>(ev, U, d, R);
+        rc = gemm_f64(d, d, d, U, d, true, R, d, false, W, d, st);
+        if (rc == LV_OK) rc = gemm_f64(d, D, d, W, d, false, A64, D, false, R, D, st);
     }
     if (rc == LV_OK) {
         f64_to_f32_k<<<(unsigned)((dD + 255) / 256), 256, 0, st>>>(R, (int64_t)dD, A);
