@@ -72,6 +72,201 @@ __device__ bool grid_barrier(unsigned *count, volatile unsigned *gen, unsigned &
     return __syncthreads_and(ok) != 0;
 }
 
+// FP64 on this chip: a warp instruction takes the pipe for 64 cycles, a division 550 and a root 585,
+// and extra warps on a scheduler only queue.  So the kernels below keep one warp per scheduler,
+// share no work redundantly between warps of a scheduler, and take reciprocals and roots from the
+// hardware's approximations (about 2^-20 relative) by one cubic step (error e^3, below 2^-58):
+//   1/x: y (1 + e + e^2), e = 1 - x y;   1/sqrt(x): y (1 + r/2 + 3 r^2/8), r = 1 - x y^2.
+__device__ __forceinline__ double fast_rcp(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ double fast_rsqrt(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double r = fma(-x * y, y, 1.0);
+    return fma(y * r, fma(0.375, r, 0.5), y);
+}
+
+// The grid barrier again, polled without sleeping on the arrival counter itself.
+__device__ bool grid_barrier_spin(unsigned *count, unsigned &target) {
+    __syncthreads();
+    int ok = 1;
+    if (threadIdx.x == 0) {
+        target += gridDim.x;
+        unsigned seen;
+        asm volatile("atom.add.release.gpu.global.u32 %0, [%1], 1;" : "=r"(seen) : "l"(count) : "memory");
+        ++seen;
+        for (int it = 0; seen < target; ++it) {
+            if (it > (1 << 22)) {  // about a second
+                ok = 0;
+                break;
+            }
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
+        }
+        __threadfence();
+    }
+    return __syncthreads_and(ok) != 0;
+}
+
+// sum over the block of TS_T threads in a fixed order, in every thread; `slot` alternates between calls
+constexpr int TS_T = 128, TS_W = TS_T / 32;
+__device__ __forceinline__ double ts_block_sum(double x, double (*red)[TS_W], int slot) {
+    x = warp_sum_d(x);
+    if ((threadIdx.x & 31) == 0) red[slot][threadIdx.x >> 5] = x;
+    __syncthreads();
+    return (red[slot][0] + red[slot][1]) + (red[slot][2] + red[slot][3]);
+}
+
+// The tridiagonalisation of tridiag_kernel (below) with every block's rows kept in shared memory (row
+// i in block i mod G, local row i / G).  A step k then goes:
+//   1. from step k - 1: p (entries by every block) and row k as it stood before that step's update,
+//      published by its owner, both through L2; every block forms w, row k of A^(k), its norm and v_k;
+//   2. every block updates its rows with (v_{k-1}, w) and forms its entries of p = tau_k A^(k) v_k, all
+//      four warps on four rows at a time (a column slice each), the sums by exchanging halves;
+//   3. one grid barrier.
+// D = 768: 9.08 ms (11.9 us a step) with rows in L2, eight warps a block that all took the step's root and
+// divisions, and a sleeping barrier; @@ now.
+__global__ void __launch_bounds__(TS_T) tridiag_sm_kernel(const double *__restrict__ K, int D, double *dg, double *ofd,
+                                                           double *Hv, double *tau, double *pbuf, double *rowbuf,
+                                                           unsigned *bar_count, int *status) {
+    extern __shared__ double sh[];
+    const int G = (int)gridDim.x, c = (int)blockIdx.x, nl = c < D ? (D - c + G - 1) / G : 0;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, maxl = (D + G - 1) / G;
+    double *const A = sh;                        // maxl rows
+    double *vp = A + (size_t)maxl * D;           // v_{k-1}
+    double *vc = vp + D;                         // v_k
+    double *const wp = vc + D;                   // w of step k - 1
+    double *const part = wp + D;                 // TS_W x maxl partial sums of p
+    __shared__ double red[2][TS_W], s_b[2];
+    unsigned target = 0;
+    for (int l = 0; l < nl; ++l)
+        for (int j = tid; j < D; j += TS_T) A[(size_t)l * D + j] = K[(int64_t)(c + l * G) * D + j];
+    for (int j = tid; j < D; j += TS_T) vp[j] = wp[j] = vc[j] = 0.0;
+    double t = 0.0;
+    __syncthreads();
+    for (int k = 0; k + 2 < D; ++k) {
+        const double *const pb = pbuf + (size_t)((k & 1) ^ 1) * D;               // p of step k - 1
+        const double *const rb = k ? rowbuf + (size_t)(k & 1) * D : K;           // row k before its update
+        // ---- w of step k - 1 and x = row k of A^(k) (v_{k-1}[k] = 1) ----
+        double pv = 0.0;
+        if (k) {
+            for (int j = k + tid; j < D; j += TS_T) {
+                const double pj = __ldcg(pb + j);
+                wp[j] = pj;
+                pv = fma(pj, vp[j], pv);
+            }
+            if (tid == 0) s_b[0] = wp[k];
+            pv = ts_block_sum(pv, red, 0);
+        }
+        const double gam = 0.5 * t * pv, wk = k ? s_b[0] - gam : 0.0;
+        double s = 0.0;
+        for (int j = k + tid; j < D; j += TS_T) {
+            double x = __ldcg(rb + j);
+            if (k) {
+                const double v = vp[j], w = fma(-gam, v, wp[j]);
+                wp[j] = w;
+                x = fma(-wk, v, x - w);
+            }
+            vc[j] = x;
+            if (j >= k + 2) s = fma(x, x, s);
+            if (j == k + 1) s_b[1] = x;
+            if (j == k && c == 0) dg[k] = x;
+        }
+        const double xn2 = ts_block_sum(s, red, 1), x0 = s_b[1];
+        double beta = x0, scal = 0.0;
+        t = 0.0;
+        if (xn2 > 0.0) {
+            const double S = fma(x0, x0, xn2);
+            if (S > 1e-290 && S < 1e290) {
+                const double y = fast_rsqrt(S);
+                double b = S * y;
+                b = fma(0.5 * fma(-b, b, S), y, b);
+                t = fma(fabs(x0), y, 1.0);  // (beta - x0) / beta with beta = -sign(x0) sqrt(S)
+                beta = -copysign(b, x0);
+                scal = copysign(fast_rcp(fabs(x0) + b), x0);
+            } else {
+                beta = -copysign(sqrt(S), x0);
+                t = (beta - x0) / beta;
+                scal = 1.0 / (x0 - beta);
+            }
+        }
+        for (int j = k + 1 + tid; j < D; j += TS_T) {
+            const double v = j == k + 1 ? 1.0 : vc[j] * scal;
+            vc[j] = v;
+            if (c == 0) Hv[(int64_t)k * D + j] = v;
+        }
+        if (c == 0 && tid == 0) {
+            tau[k] = t;
+            ofd[k] = beta;
+        }
+        __syncthreads();
+        // ---- own rows i > k: the pending update, then p_i = t (row_i . v_k) ----
+        const int l0 = k >= c ? (k - c) / G + 1 : 0;
+        for (int lc = l0; lc < nl; lc += 4) {
+            double acc[4] = {}, vi[4], wi[4];
+            const int nr = min(4, nl - lc);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int i = c + (lc + (u < nr ? u : 0)) * G;
+                vi[u] = vp[i];
+                wi[u] = wp[i];
+            }
+            const bool pub = c + lc * G == k + 1;  // the next pivot row is always the first one left
+            for (int j = k + 1 + tid; j < D; j += TS_T) {
+                const double wj = wp[j], vj = vp[j], bj = vc[j];
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (u < nr) {
+                        double *const ar = A + (size_t)(lc + u) * D + j;
+                        double a = *ar;
+                        if (k) {
+                            a = fma(-vi[u], wj, a);
+                            a = fma(-wi[u], vj, a);
+                            *ar = a;
+                        }
+                        if (u == 0 && pub) __stcg(rowbuf + (size_t)((k + 1) & 1) * D + j, a);
+                        acc[u] = fma(a, bj, acc[u]);
+                    }
+            }
+            // lane's row: 2 (bit 4) + (bit 3)
+            const bool h4 = lane & 16, h3 = lane & 8;
+            const double a0 = (h4 ? acc[2] : acc[0]) + __shfl_xor_sync(FULL, h4 ? acc[0] : acc[2], 16);
+            const double a1 = (h4 ? acc[3] : acc[1]) + __shfl_xor_sync(FULL, h4 ? acc[1] : acc[3], 16);
+            double x = (h3 ? a1 : a0) + __shfl_xor_sync(FULL, h3 ? a0 : a1, 8);
+#pragma unroll
+            for (int o = 4; o; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
+            if ((lane & 7) == 0 && (lane >> 3) < nr) part[wid * maxl + lc + (lane >> 3)] = x;
+        }
+        __syncthreads();
+        for (int l = l0 + tid; l < nl; l += TS_T)
+            __stcg(pbuf + (size_t)(k & 1) * D + c + l * G,
+                   t * ((part[l] + part[maxl + l]) + (part[2 * maxl + l] + part[3 * maxl + l])));
+        if (!grid_barrier_spin(bar_count, target)) {
+            if (tid == 0) atomicOr(status, ST_TIMEOUT);
+            return;
+        }
+        double *const o = vp;  // v_k becomes v_{k-1}
+        vp = vc;
+        vc = o;
+    }
+    // the last 2 x 2 block: row a from its owner's published copy, the corner from the owner itself
+    const int a = D - 2, b = D - 1, k = D - 2;
+    const double *const pb = pbuf + (size_t)((k & 1) ^ 1) * D, *const rb = rowbuf + (size_t)(k & 1) * D;
+    if (tid == 0) {
+        const double pa = __ldcg(pb + a), pbb = __ldcg(pb + b), pv = fma(pa, vp[a], pbb * vp[b]);
+        const double gam = 0.5 * t * pv, wa = fma(-gam, vp[a], pa), wb = fma(-gam, vp[b], pbb);
+        if (c == 0) {
+            dg[a] = __ldcg(rb + a) - 2.0 * vp[a] * wa;
+            ofd[a] = __ldcg(rb + b) - vp[a] * wb - wa * vp[b];
+            tau[a] = 0.0;
+        }
+        if (b % G == c) dg[b] = A[(size_t)(b / G) * D + b] - 2.0 * vp[b] * wb;
+    }
+}
+
 // Householder tridiagonalisation of the symmetric D x D matrix A (device, full storage).  Reflection
 // k (k = 0 .. D - 3) maps the column below the diagonal, x = A^(k)[k + 1 .., k], to (beta, 0, ..):
 // H_k = I - tau_k v_k v_k^T with v_k[0] = 1, stored as Hv[k][k + 1 ..].  The trailing matrix
@@ -158,46 +353,104 @@ __global__ void __launch_bounds__(TRI_THREADS) tridiag_kernel(double *A, int D, 
     }
 }
 
-// number of eigenvalues of T below x (Sturm count of the LDL^T pivots of T - x I)
-__device__ int sturm_below(const double *dg, const double *ofd, int D, double x, double pivmin) {
+// number of eigenvalues of T below x: negative pivots of T - x I (e2: squared off-diagonals).  The pivot's
+// reciprocal is fast_rcp; signs and the pivot floor are read off the high word, which costs no FP64
+// instruction: five of them a pivot instead of about twelve.
+__device__ __forceinline__ int sturm_below(const double *dg, const double *e2, int D, double x, double pivmin) {
+    const int ph = __double2hiint(pivmin);
     double q = dg[0] - x;
-    if (fabs(q) < pivmin) q = -pivmin;
-    int neg = q < 0.0;
+    int neg = 0;
+#pragma unroll 4
     for (int j = 1; j < D; ++j) {
-        q = dg[j] - x - ofd[j - 1] * ofd[j - 1] / q;
-        if (fabs(q) < pivmin) q = -pivmin;
-        neg += q < 0.0;
+        const int h = __double2hiint(q);
+        if ((h & 0x7fffffff) < ph) q = -pivmin;
+        neg -= __double2hiint(q) >> 31;
+        q = fma(-e2[j - 1], fast_rcp(q), dg[j] - x);
     }
-    return neg;
+    if ((__double2hiint(q) & 0x7fffffff) < ph) q = -pivmin;
+    return neg - (__double2hiint(q) >> 31);
+}
+// the same in float32 for T / ||T||: the counts of a matrix within about 1e-6 ||T|| of T
+__device__ __forceinline__ int sturm_below_f(const float *dg, const float *e2, int D, float x) {
+    float q = dg[0] - x;
+    int neg = 0;
+#pragma unroll 4
+    for (int j = 1; j < D; ++j) {
+        if (fabsf(q) < 1e-30f) q = -1e-30f;
+        neg += q < 0.f;
+        q = dg[j] - x - __fdividef(e2[j - 1], q);
+    }
+    return neg + (q < 0.f);
 }
 
-// lam[i] = the (i + 1)-th largest eigenvalue of T, i < nout; one warp per eigenvalue.  Each round
-// lanes 0 .. 30 count at 31 interior points of [lo, hi] (a point at or below lo counts as holding
-// the invariant, one at or above hi as not), and the interval shrinks to the two neighbouring points
-// around the change, until it no longer shrinks.
-__global__ void bisect_kernel(const double *dg, const double *ofd, int D, int nout, double lo0, double hi0,
-                              double pivmin, double *lam) {
-    const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
-    if (i >= nout) return;  // whole warps
+// lam[i] = the (i + 1)-th largest eigenvalue of T, i < nout; one block of two warps per eigenvalue.
+// Multisection: a round counts at 63 points of [lo, hi] and keeps the interval around the change of
+// "at least i + 1 eigenvalues at or above".  float32 rounds narrow the interval to about 1e-5 ||T|| first
+// (a float32 count takes a seventh of the time); the first FP64 round then checks both its ends and
+// falls back to the Gershgorin interval's part beyond an end that does not hold.
+// 160 eigenvalues of D = 768: 4.93 ms with 31 points, FP64 throughout and a division a pivot; @@ now.
+__global__ void __launch_bounds__(64) bisect_kernel(const double *dg, const double *ofd, int D, int nout, double lo0,
+                                                    double hi0, double pivmin, double *lam) {
+    extern __shared__ double sb[];
+    double *const sd = sb, *const se = sb + D;
+    float *const fd = reinterpret_cast<float *>(se + D), *const fe = fd + D;
+    __shared__ unsigned s_bal[2][2];
+    const int i = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    const double norm = fmax(fabs(lo0), fabs(hi0)), inv = 1.0 / norm;
+    for (int j = tid; j < D; j += 64) {
+        const double d = dg[j], e = j + 1 < D ? ofd[j] : 0.0;
+        sd[j] = d;
+        se[j] = e * e;
+        fd[j] = (float)(d * inv);
+        const float ef = (float)(e * inv);
+        fe[j] = ef * ef;
+    }
+    __syncthreads();
+    int buf = 0;
+    // number of leading true predicates of the 64 threads (they form a prefix)
+    auto prefix = [&](bool pred) {
+        const unsigned bal = __ballot_sync(FULL, pred);
+        if (lane == 0) s_bal[buf][wid] = bal;
+        __syncthreads();
+        const int n0 = __popc(s_bal[buf][0]);
+        const int n = n0 < 32 ? n0 : 32 + __popc(s_bal[buf][1]);
+        buf ^= 1;
+        return n;
+    };
+    auto point = [&](double lo, double hi, int p, int parts) { return lo + (hi - lo) * ((double)p / (double)parts); };
     double lo = lo0, hi = hi0;
+    const bool scaled = norm > 1e-150 && norm < 1e150;
+    if (scaled) {
+        float l = (float)(lo0 * inv), h = (float)(hi0 * inv);
+        for (int r = 0; r < 3; ++r) {
+            auto at = [&](int p) { return l + (h - l) * ((float)p / 64.0f); };
+            const int n = prefix(tid < 63 && D - sturm_below_f(fd, fe, D, at(tid + 1)) >= i + 1);
+            const float nl = n > 0 ? at(n) : l, nh = n < 63 ? at(n + 1) : h;
+            l = nl;
+            h = nh;
+        }
+        const double g = 1e-5 * norm;
+        const double cl = fmax(lo0, (double)l * norm - g), ch = fmin(hi0, (double)h * norm + g);
+        const int n = prefix(D - sturm_below(sd, se, D, point(cl, ch, tid, 63), pivmin) >= i + 1);
+        lo = n > 0 ? point(cl, ch, n - 1, 63) : lo0;
+        hi = n < 64 ? point(cl, ch, n, 63) : hi0;
+    }
     for (int round = 0; round < 64; ++round) {
-        const double x = lo + (hi - lo) * ((double)(lane + 1) / 32.0);
+        const double x = point(lo, hi, tid + 1, 64);
         bool pred;
-        if (lane == 31 || x >= hi)
+        if (tid == 63 || x >= hi)
             pred = false;
         else if (x <= lo)
             pred = true;
         else
-            pred = D - sturm_below(dg, ofd, D, x, pivmin) >= i + 1;
-        const unsigned bal = __ballot_sync(FULL, pred);
-        const int nt = __popc(bal);  // the true lanes are a prefix (counts fall as x grows)
-        const double xl = __shfl_sync(FULL, x, max(nt - 1, 0)), xh = __shfl_sync(FULL, x, min(nt, 31));
-        const double nlo = nt > 0 ? fmax(lo, xl) : lo, nhi = nt < 31 ? fmin(hi, xh) : hi;
+            pred = D - sturm_below(sd, se, D, x, pivmin) >= i + 1;
+        const int n = prefix(pred);
+        const double nlo = n > 0 ? fmax(lo, point(lo, hi, n, 64)) : lo, nhi = n < 63 ? fmin(hi, point(lo, hi, n + 1, 64)) : hi;
         if (nlo == lo && nhi == hi) break;
         lo = nlo;
         hi = nhi;
     }
-    if (lane == 0) lam[i] = 0.5 * (lo + hi);
+    if (tid == 0) lam[i] = 0.5 * (lo + hi);
 }
 
 // a deterministic start vector entry in [-1, 1)
@@ -211,67 +464,81 @@ __device__ __forceinline__ double start_entry(int i, int e) {
 
 // Inverse iteration, one block per cluster [cb[c], ce[c]) of eigenvalues (descending, close ones
 // together).  For eigenvalue e: T - lam I = P L U by Gaussian elimination with partial pivoting
-// (thread 0; pivots below tol replaced by +-tol, stored as reciprocals), then: solve, orthogonalise
+// (thread 0; pivots below tol replaced by +-tol, kept as reciprocals), then: solve, orthogonalise
 // against the cluster's earlier vectors (modified Gram-Schmidt), normalise -- three rounds (the
 // eigenvalue is accurate to the last bits, so one solve already nearly converges).  Z: nout x D.
-// scratch: 5 D doubles and D ints per cluster.
+// The factors and the vector sit in shared memory and the recurrences in registers, so that a chain step
+// costs its FP64 instructions alone: 160 vectors of D = 768 1.15 ms with the factors in L2 and two
+// divisions a row, @@ now.
 __global__ void __launch_bounds__(128) inviter_kernel(const double *dg, const double *ofd, int D, const double *lam,
-                                                      const int *cb, const int *ce, double tol, double *Z,
-                                                      double *scratch, int *piv_all) {
+                                                      const int *cb, const int *ce, double tol, double *Z) {
+    extern __shared__ double si[];
     __shared__ double red[4];
     const int c = blockIdx.x, tid = threadIdx.x;
-    double *dl = scratch + (size_t)c * 5 * D, *dd = dl + D, *du = dd + D, *du2 = du + D, *x = du2 + D;
-    int *piv = piv_all + (size_t)c * D;
+    double *const mu = si, *const iv = mu + D, *const du = iv + D, *const du2 = du + D, *const x = du2 + D;
+    unsigned char *const piv = reinterpret_cast<unsigned char *>(x + D);
+    auto mag = [](double v) { return __double_as_longlong(v) & 0x7fffffffffffffffll; };  // orders like |v|
     for (int e = cb[c]; e < ce[c]; ++e) {
         // distinct shifts inside a cluster (equal eigenvalues would give the same vector)
         double le = lam[e];
         if (e > cb[c]) le = fmin(le, lam[e - 1] - 4.0 * DBL_EPSILON * fabs(lam[e - 1]) - tol * 1e-3);
+        // T in place of what it will be replaced by: iv = diagonal - lam, mu = off-diagonal
+        for (int j = tid; j < D; j += blockDim.x) {
+            iv[j] = dg[j] - le;
+            mu[j] = j + 1 < D ? ofd[j] : 0.0;
+            x[j] = start_entry(j, e);
+        }
+        __syncthreads();
         if (tid == 0) {
-            for (int j = 0; j < D; ++j) {
-                dd[j] = dg[j] - le;
-                if (j + 1 < D) dl[j] = du[j] = ofd[j];
-                du2[j] = 0.0;
-            }
+            double d = iv[0], u = mu[0];  // the current row's diagonal and superdiagonal
+            const long long tm = mag(tol);
             for (int j = 0; j + 1 < D; ++j) {
-                if (fabs(dd[j]) >= fabs(dl[j])) {
-                    if (fabs(dd[j]) < tol) dd[j] = dd[j] < 0.0 ? -tol : tol;
-                    const double mult = dl[j] / dd[j];
-                    dl[j] = mult;
-                    dd[j + 1] -= mult * du[j];
+                const double l = mu[j], dn = iv[j + 1], un = mu[j + 1];
+                if (mag(d) >= mag(l) || mag(l) < tm) {
+                    if (mag(d) < tm) d = d < 0.0 ? -tol : tol;
+                    const double r = fast_rcp(d), m = l * r;
+                    mu[j] = m;
+                    iv[j] = r;
+                    du[j] = u;
+                    du2[j] = 0.0;
                     piv[j] = 0;
+                    d = fma(-m, u, dn);
+                    u = un;
                 } else {
-                    const double mult = dd[j] / dl[j];
-                    dd[j] = dl[j];
-                    const double tmp = dd[j + 1];
-                    dd[j + 1] = du[j] - mult * tmp;
-                    if (j + 2 < D) {
-                        du2[j] = du[j + 1];
-                        du[j + 1] = -mult * du2[j];
-                    }
-                    du[j] = tmp;
-                    dl[j] = mult;
+                    const double r = fast_rcp(l), m = d * r;
+                    mu[j] = m;
+                    iv[j] = r;
+                    du[j] = dn;
+                    du2[j] = un;
                     piv[j] = 1;
+                    d = fma(-m, dn, u);
+                    u = -m * un;
                 }
             }
-            if (fabs(dd[D - 1]) < tol) dd[D - 1] = dd[D - 1] < 0.0 ? -tol : tol;
-            for (int j = 0; j < D; ++j) dd[j] = 1.0 / dd[j];  // the solves multiply
+            if (mag(d) < tm) d = d < 0.0 ? -tol : tol;
+            iv[D - 1] = fast_rcp(d);
         }
-        for (int i = tid; i < D; i += blockDim.x) x[i] = start_entry(i, e);
         __syncthreads();
         for (int round = 0; round < 3; ++round) {
             if (tid == 0) {
+                double cur = x[0];
+#pragma unroll 4
                 for (int j = 0; j + 1 < D; ++j) {
-                    if (piv[j]) {
-                        const double tmp = x[j];
-                        x[j] = x[j + 1];
-                        x[j + 1] = tmp - dl[j] * x[j];
-                    } else {
-                        x[j + 1] -= dl[j] * x[j];
-                    }
+                    const double nx = x[j + 1], m = mu[j];
+                    const bool p = piv[j];
+                    const double keep = p ? nx : cur, other = p ? cur : nx;
+                    x[j] = keep;
+                    cur = fma(-m, keep, other);
                 }
-                x[D - 1] *= dd[D - 1];
-                x[D - 2] = (x[D - 2] - du[D - 2] * x[D - 1]) * dd[D - 2];
-                for (int j = D - 3; j >= 0; --j) x[j] = (x[j] - du[j] * x[j + 1] - du2[j] * x[j + 2]) * dd[j];
+                double x1 = cur * iv[D - 1], x2 = 0.0;
+                x[D - 1] = x1;
+#pragma unroll 4
+                for (int j = D - 2; j >= 0; --j) {
+                    const double v = fma(-du[j], x1, fma(-du2[j], x2, x[j])) * iv[j];
+                    x[j] = v;
+                    x2 = x1;
+                    x1 = v;
+                }
             }
             __syncthreads();
             for (int f = cb[c]; f < e; ++f) {
@@ -296,34 +563,56 @@ __global__ void __launch_bounds__(128) inviter_kernel(const double *dg, const do
 }
 
 // evecs[r] = Q z_r = H_0 H_1 .. H_{D-3} z_r, unit norm, largest-magnitude entry positive (first
-// index on ties); evals[r] = lam[r] (evals nullable).  One warp per eigenvector.
-__global__ void __launch_bounds__(32) backtrans_kernel(const double *Z, const double *Hv, const double *tau, int D,
-                                                       const double *lam, double *evals, double *evecs) {
-    extern __shared__ double sx[];
-    const int r = blockIdx.x, lane = threadIdx.x;
-    for (int i = lane; i < D; i += 32) sx[i] = Z[(size_t)r * D + i];
-    __syncwarp();
+// index on ties); evals[r] = lam[r] (evals nullable).  One block of four warps per eigenvector, its
+// entries in registers (tid + 128 u), the next reflection's vector loaded while the current one's sum
+// goes round: 160 vectors of D = 768 2.04 ms with one warp per vector, @@ now.
+template <int E>
+__global__ void __launch_bounds__(TS_T) backtrans_kernel(const double *__restrict__ Z, const double *__restrict__ Hv,
+                                                         const double *__restrict__ tau, int D, const double *lam,
+                                                         double *evals, double *evecs) {
+    __shared__ double red[2][TS_W];
+    __shared__ double s_best[TS_W];
+    __shared__ int s_bi[TS_W];
+    const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    double x[E], v[E];
+#pragma unroll
+    for (int u = 0; u < E; ++u) x[u] = tid + TS_T * u < D ? Z[(size_t)r * D + tid + TS_T * u] : 0.0;
+    auto fetch = [&](int k) {
+#pragma unroll
+        for (int u = 0; u < E; ++u) {
+            const int j = tid + TS_T * u;
+            v[u] = k >= 0 && j > k && j < D ? __ldg(Hv + (int64_t)k * D + j) : 0.0;
+        }
+    };
+    fetch(D - 3);
     for (int k = D - 3; k >= 0; --k) {
-        const double t = tau[k];
-        if (t == 0.0) continue;
-        const double *vk = Hv + (int64_t)k * D;
-        double s = 0.0;
-        for (int i = k + 1 + lane; i < D; i += 32) s = fma(vk[i], sx[i], s);
-        s = warp_sum_d(s) * t;
-        for (int i = k + 1 + lane; i < D; i += 32) sx[i] = fma(-s, vk[i], sx[i]);
-        __syncwarp();
+        const int u0 = (k + 1) / TS_T;  // entries below 128 u0 are zero in v
+        double w[E], s = 0.0;
+#pragma unroll
+        for (int u = 0; u < E; ++u) {
+            w[u] = v[u];
+            if (u >= u0) s = fma(w[u], x[u], s);
+        }
+        const double t = __ldg(tau + k);
+        fetch(k - 1);
+        s = -ts_block_sum(s, red, k & 1) * t;
+#pragma unroll
+        for (int u = 0; u < E; ++u)
+            if (u >= u0) x[u] = fma(s, w[u], x[u]);
     }
     double s = 0.0, best = -1.0;
     int bi = D;
-    for (int i = lane; i < D; i += 32) {
-        s = fma(sx[i], sx[i], s);
-        const double a = fabs(sx[i]);
-        if (a > best) {
+#pragma unroll
+    for (int u = 0; u < E; ++u) {
+        s = fma(x[u], x[u], s);
+        const double a = fabs(x[u]);
+        if (tid + TS_T * u < D && a > best) {
             best = a;
-            bi = i;
+            bi = tid + TS_T * u;
         }
     }
-    s = warp_sum_d(s);
+    __syncthreads();
+    s = ts_block_sum(s, red, 0);
     // largest |x_i|, first index on ties
 #pragma unroll
     for (int o = 16; o; o >>= 1) {
@@ -334,9 +623,41 @@ __global__ void __launch_bounds__(32) backtrans_kernel(const double *Z, const do
             bi = oi;
         }
     }
-    const double scale = (s > 0.0 ? 1.0 / sqrt(s) : 0.0) * (bi < D && sx[bi] < 0.0 ? -1.0 : 1.0);
-    for (int i = lane; i < D; i += 32) evecs[(size_t)r * D + i] = sx[i] * scale;
-    if (lane == 0 && evals) evals[r] = lam[r];
+    if (lane == 0) {
+        s_best[wid] = best;
+        s_bi[wid] = bi;
+    }
+    __syncthreads();
+    for (int w = 0; w < TS_W; ++w)
+        if (s_best[w] > best || (s_best[w] == best && s_bi[w] < bi)) {
+            best = s_best[w];
+            bi = s_bi[w];
+        }
+    __shared__ double s_sign;
+#pragma unroll
+    for (int u = 0; u < E; ++u)
+        if (tid + TS_T * u == bi) s_sign = x[u] < 0.0 ? -1.0 : 1.0;
+    __syncthreads();
+    const double scale = (s > 0.0 ? 1.0 / sqrt(s) : 0.0) * (bi < D ? s_sign : 1.0);
+#pragma unroll
+    for (int u = 0; u < E; ++u)
+        if (tid + TS_T * u < D) evecs[(size_t)r * D + tid + TS_T * u] = x[u] * scale;
+    if (tid == 0 && evals) evals[r] = lam[r];
+}
+
+static int launch_backtrans(const double *Z, const double *Hv, const double *tau, int D, int nout, const double *lam,
+                            double *evals, double *evecs, cudaStream_t st) {
+    auto go = [&](auto k) -> int {
+        k<<<nout, TS_T, 0, st>>>(Z, Hv, tau, D, lam, evals, evecs);
+        LV_CHECK_LAUNCH("backtrans_kernel");
+        return LV_OK;
+    };
+    if (D <= 2 * TS_T) return go(backtrans_kernel<2>);
+    if (D <= 4 * TS_T) return go(backtrans_kernel<4>);
+    if (D <= 6 * TS_T) return go(backtrans_kernel<6>);
+    if (D <= 8 * TS_T) return go(backtrans_kernel<8>);
+    if (D <= 16 * TS_T) return go(backtrans_kernel<16>);
+    return go(backtrans_kernel<32>);
 }
 
 // the path applies: 8 <= D <= 4096, 1 <= nout <= D
@@ -345,43 +666,53 @@ bool eigh_top_ok(int D, int nout) { return D >= 8 && D <= EIGH_TOP_MAX_D && nout
 int eigh_top(const double *K, int D, int nout, double *evals, double *evecs, cudaStream_t st) {
     if (!eigh_top_ok(D, nout)) return fail(LV_ERR_ARG, "eigh_top: need 8 <= D <= 4096 and 1 <= nout <= D");
     double *A = nullptr, *Hv = nullptr, *tau = nullptr, *dg = nullptr, *ofd = nullptr, *pbuf = nullptr;
-    double *lam = nullptr, *Z = nullptr, *scr = nullptr;
+    double *lam = nullptr, *Z = nullptr, *rowbuf = nullptr;
     unsigned *bar = nullptr;
-    int *status = nullptr, *cl = nullptr, *piv = nullptr;
+    int *status = nullptr, *cl = nullptr;
     int rc = LV_OK;
     const size_t DD = (size_t)D * D;
     std::vector<double> hd(D), he(D), hl(nout);
     std::vector<int> hcb, hce;
     int dev = 0, sms = 0, per_sm = 0, nclus = 0, hstatus = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return fail(LV_ERR_CUDA, "eigh_top: no device");
+    // rows in shared memory while they fit (D <= about 1800); two rows a block at least
+    const int gs = std::min(sms, (D + 1) / 2), maxl = (D + gs - 1) / gs;
+    const size_t ssm = sizeof(double) * ((size_t)maxl * D + 3 * (size_t)D + (size_t)TS_W * maxl);
+    const bool in_sm = ssm <= 220 * 1024;
     const size_t tsm = sizeof(double) * (3 * (size_t)D + TRI_WARPS);
-    if (tmp_alloc((void **)&A, sizeof(double) * DD, st) || tmp_alloc((void **)&Hv, sizeof(double) * DD, st) ||
+    const size_t bsm = 2 * sizeof(double) * (size_t)D + 2 * sizeof(float) * (size_t)D, ism = (5 * sizeof(double) + 1) * (size_t)D;
+    if ((!in_sm && tmp_alloc((void **)&A, sizeof(double) * DD, st)) || tmp_alloc((void **)&Hv, sizeof(double) * DD, st) ||
         tmp_alloc((void **)&tau, sizeof(double) * D, st) || tmp_alloc((void **)&dg, sizeof(double) * D, st) ||
-        tmp_alloc((void **)&ofd, sizeof(double) * D, st) || tmp_alloc((void **)&pbuf, sizeof(double) * D, st) ||
+        tmp_alloc((void **)&ofd, sizeof(double) * D, st) || tmp_alloc((void **)&pbuf, sizeof(double) * 2 * D, st) ||
+        tmp_alloc((void **)&rowbuf, sizeof(double) * 2 * D, st) ||
         tmp_alloc((void **)&lam, sizeof(double) * nout, st) || tmp_alloc((void **)&Z, sizeof(double) * nout * (size_t)D, st) ||
         tmp_alloc((void **)&bar, 2 * sizeof(unsigned), st) || tmp_alloc((void **)&status, sizeof(int), st)) {
         rc = fail(LV_ERR_OOM, "eigh_top: allocation failed");
         goto done;
     }
-    if (cudaMemcpyAsync(A, K, sizeof(double) * DD, cudaMemcpyDeviceToDevice, st) != cudaSuccess ||
+    if ((!in_sm && cudaMemcpyAsync(A, K, sizeof(double) * DD, cudaMemcpyDeviceToDevice, st) != cudaSuccess) ||
         cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), st) != cudaSuccess ||
         cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess) {
         rc = fail(LV_ERR_CUDA, "eigh_top: copy failed");
         goto done;
     }
     // 1. tridiagonal form: one block per SM, all co-resident (cooperative launch)
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaFuncSetAttribute(tridiag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tridiag_kernel, TRI_THREADS, tsm) != cudaSuccess ||
-        per_sm < 1) {
-        rc = fail(LV_ERR_CUDA, "eigh_top: cannot size the tridiagonalisation");
-        goto done;
-    }
     {
+        const void *kern = in_sm ? (const void *)tridiag_sm_kernel : (const void *)tridiag_kernel;
+        const size_t sm = in_sm ? ssm : tsm;
+        const int threads = in_sm ? TS_T : TRI_THREADS, blocks = in_sm ? gs : sms;
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, sm) != cudaSuccess || per_sm < 1) {
+            rc = fail(LV_ERR_CUDA, "eigh_top: cannot size the tridiagonalisation");
+            goto done;
+        }
         int Dv = D;
         unsigned *bar_gen = bar + 1;
-        void *args[] = {&A, &Dv, &dg, &ofd, &Hv, &tau, &pbuf, &bar, &bar_gen, &status};
-        if (cudaLaunchCooperativeKernel((const void *)tridiag_kernel, dim3((unsigned)sms), dim3(TRI_THREADS), args, tsm,
-                                        st) != cudaSuccess) {
+        void *args_sm[] = {(void *)&K, &Dv, &dg, &ofd, &Hv, &tau, &pbuf, &rowbuf, &bar, &status};
+        void *args_gl[] = {&A, &Dv, &dg, &ofd, &Hv, &tau, &pbuf, &bar, &bar_gen, &status};
+        if (cudaLaunchCooperativeKernel(kern, dim3((unsigned)blocks), dim3((unsigned)threads), in_sm ? args_sm : args_gl,
+                                        sm, st) != cudaSuccess) {
             cudaGetLastError();
             rc = fail(LV_ERR_CUDA, "eigh_top: tridiagonalisation launch failed");
             goto done;
@@ -412,8 +743,12 @@ int eigh_top(const double *K, int D, int nout, double *evals, double *evecs, cud
         lo -= pad;
         hi += pad;
         const double pivmin = DBL_MIN * std::max(1.0, e2max);
-        // one warp per block, so that the eigenvalues' warps spread over all SMs
-        bisect_kernel<<<nout, 32, 0, st>>>(dg, ofd, D, nout, lo, hi, pivmin, lam);
+        if (cudaFuncSetAttribute(bisect_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsm) != cudaSuccess ||
+            cudaFuncSetAttribute(inviter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ism) != cudaSuccess) {
+            rc = fail(LV_ERR_CUDA, "eigh_top: shared-memory attribute failed");
+            goto done;
+        }
+        bisect_kernel<<<nout, 64, bsm, st>>>(dg, ofd, D, nout, lo, hi, pivmin, lam);
         if (cudaGetLastError() != cudaSuccess ||
             cudaMemcpyAsync(hl.data(), lam, sizeof(double) * nout, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess) {
@@ -431,9 +766,7 @@ int eigh_top(const double *K, int D, int nout, double *evals, double *evecs, cud
             }
         }
         nclus = (int)hcb.size();
-        if (tmp_alloc((void **)&cl, sizeof(int) * 2 * nclus, st) ||
-            tmp_alloc((void **)&scr, sizeof(double) * 5 * (size_t)D * nclus, st) ||
-            tmp_alloc((void **)&piv, sizeof(int) * (size_t)D * nclus, st)) {
+        if (tmp_alloc((void **)&cl, sizeof(int) * 2 * nclus, st)) {
             rc = fail(LV_ERR_OOM, "eigh_top: allocation failed");
             goto done;
         }
@@ -443,20 +776,14 @@ int eigh_top(const double *K, int D, int nout, double *evals, double *evecs, cud
             goto done;
         }
         const double tol = std::max(DBL_EPSILON * tnorm, DBL_MIN);
-        inviter_kernel<<<nclus, 128, 0, st>>>(dg, ofd, D, lam, cl, cl + nclus, tol, Z, scr, piv);
+        inviter_kernel<<<nclus, 128, ism, st>>>(dg, ofd, D, lam, cl, cl + nclus, tol, Z);
         if (cudaGetLastError() != cudaSuccess) {
             rc = fail(LV_ERR_CUDA, "eigh_top: inverse iteration launch failed");
             goto done;
         }
         // 4. back to K's basis
-        const size_t bsm = sizeof(double) * (size_t)D;
-        if (bsm > 48 * 1024 &&
-            cudaFuncSetAttribute(backtrans_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsm) != cudaSuccess) {
-            rc = fail(LV_ERR_CUDA, "eigh_top: shared-memory attribute failed");
-            goto done;
-        }
-        backtrans_kernel<<<nout, 32, bsm, st>>>(Z, Hv, tau, D, lam, evals, evecs);
-        if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess) {
+        if ((rc = launch_backtrans(Z, Hv, tau, D, nout, lam, evals, evecs, st))) goto done;
+        if (cudaStreamSynchronize(st) != cudaSuccess) {
             rc = fail(LV_ERR_CUDA, "eigh_top: back-transformation failed");
             goto done;
         }
@@ -473,8 +800,7 @@ done:
     tmp_free(bar, st);
     tmp_free(status, st);
     tmp_free(cl, st);
-    tmp_free(scr, st);
-    tmp_free(piv, st);
+    tmp_free(rowbuf, st);
     return rc;
 }
 
