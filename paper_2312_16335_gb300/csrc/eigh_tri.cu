@@ -3,11 +3,11 @@
 // so instead of diagonalising the whole matrix (cyclic Jacobi, fit.cu) this path
 //   1. reduces K to tridiagonal form T = Q^T K Q by D - 2 Householder reflections (one persistent
 //      kernel, all SMs, one grid barrier per reflection);
-//   2. finds the nout largest eigenvalues of T by multisection on Sturm counts (one warp each);
+//   2. finds the nout largest eigenvalues of T by multisection on Sturm counts (two warps each);
 //   3. finds their eigenvectors of T by inverse iteration on the pivoted tridiagonal factorisation
 //      of T - lambda I, with Gram-Schmidt inside clusters of close eigenvalues (one block per
 //      cluster);
-//   4. maps them back through the reflections (x = Q z, one warp per eigenvector) and fixes the
+//   4. maps them back through the reflections (x = Q z, one block per eigenvector) and fixes the
 //      sign (largest-magnitude entry positive, first index on ties).
 // FP64 throughout.  Every grid-wide wait is bounded: a block that waits too long records
 // ST_TIMEOUT and returns.
@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <cfloat>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "common.cuh"
@@ -120,15 +121,28 @@ __device__ __forceinline__ double ts_block_sum(double x, double (*red)[TS_W], in
     return (red[slot][0] + red[slot][1]) + (red[slot][2] + red[slot][3]);
 }
 
+// f(0), f(1), .. f(N - 1) with compile-time arguments.  The loops over a vector's register slots leave out
+// the slots that hold no entry any more, and they do it at compile time: an FP64 instruction whose
+// predicate is off still takes the pipe for its 64 cycles.
+template <int I = 0, int N, class F>
+__device__ __forceinline__ void phases(std::integral_constant<int, N> n, F &&f) {
+    f(std::integral_constant<int, I>());
+    if constexpr (I + 1 < N) phases<I + 1>(n, f);
+}
+
 // The tridiagonalisation of tridiag_kernel (below) with every block's rows kept in shared memory (row
-// i in block i mod G, local row i / G).  A step k then goes:
+// i in block i mod G, local row i / G) and the step's vectors in registers (entry tid + 128 u in
+// slot u, zero where the step has no entry).  A step k then goes:
 //   1. from step k - 1: p (entries by every block) and row k as it stood before that step's update,
-//      published by its owner, both through L2; every block forms w, row k of A^(k), its norm and v_k;
+//      published by its owner, both read from L2 at once; every block forms w, row k of A^(k), its
+//      norm and v_k;
 //   2. every block updates its rows with (v_{k-1}, w) and forms its entries of p = tau_k A^(k) v_k, all
-//      four warps on four rows at a time (a column slice each), the sums by exchanging halves;
+//      four warps on four rows at a time, the sums by exchanging halves;
 //   3. one grid barrier.
 // D = 768: 9.08 ms (11.9 us a step) with rows in L2, eight warps a block that all took the step's root and
-// divisions, and a sleeping barrier; @@ now.
+// divisions, and a sleeping barrier; 5.10 ms (6.7 us) now, of it about 1.2 us in the barrier, 1.7 in the
+// two sums and the root, 1.4 in the rows.
+template <int E>
 __global__ void __launch_bounds__(TS_T) tridiag_sm_kernel(const double *__restrict__ K, int D, double *dg, double *ofd,
                                                            double *Hv, double *tau, double *pbuf, double *rowbuf,
                                                            unsigned *bar_count, int *status) {
@@ -136,134 +150,176 @@ __global__ void __launch_bounds__(TS_T) tridiag_sm_kernel(const double *__restri
     const int G = (int)gridDim.x, c = (int)blockIdx.x, nl = c < D ? (D - c + G - 1) / G : 0;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, maxl = (D + G - 1) / G;
     double *const A = sh;                        // maxl rows
-    double *vp = A + (size_t)maxl * D;           // v_{k-1}
-    double *vc = vp + D;                         // v_k
-    double *const wp = vc + D;                   // w of step k - 1
-    double *const part = wp + D;                 // TS_W x maxl partial sums of p
+    double *vp_s = A + (size_t)maxl * D;         // v_{k-1}, v_k and w of step k - 1 by row, for the own rows'
+    double *vc_s = vp_s + D;                     // coefficients
+    double *const w_s = vc_s + D;
+    double *const part = w_s + D;                // TS_W x maxl partial sums of p
     __shared__ double red[2][TS_W], s_b[2];
     unsigned target = 0;
     for (int l = 0; l < nl; ++l)
         for (int j = tid; j < D; j += TS_T) A[(size_t)l * D + j] = K[(int64_t)(c + l * G) * D + j];
-    for (int j = tid; j < D; j += TS_T) vp[j] = wp[j] = vc[j] = 0.0;
+    double vp[E], vc[E], w[E], x[E];
+#pragma unroll
+    for (int u = 0; u < E; ++u) vp[u] = w[u] = 0.0;
+    for (int j = tid; j < D; j += TS_T) vp_s[j] = w_s[j] = 0.0;
     double t = 0.0;
+    bool alive = true;
     __syncthreads();
-    for (int k = 0; k + 2 < D; ++k) {
-        const double *const pb = pbuf + (size_t)((k & 1) ^ 1) * D;               // p of step k - 1
-        const double *const rb = k ? rowbuf + (size_t)(k & 1) * D : K;           // row k before its update
-        // ---- w of step k - 1 and x = row k of A^(k) (v_{k-1}[k] = 1) ----
-        double pv = 0.0;
-        if (k) {
-            for (int j = k + tid; j < D; j += TS_T) {
-                const double pj = __ldcg(pb + j);
-                wp[j] = pj;
-                pv = fma(pj, vp[j], pv);
+    // phase U0: the steps k with k / TS_T = U0; their vectors have entries in slots U0 .. E - 1
+    phases(std::integral_constant<int, E>(), [&](auto u0c) {
+        constexpr int U0 = decltype(u0c)::value;
+        const int kend = min(D - 2, TS_T * (U0 + 1));
+        for (int k = TS_T * U0; alive && k < kend; ++k) {
+            const double *const pb = pbuf + (size_t)((k & 1) ^ 1) * D;      // p of step k - 1
+            const double *const rb = k ? rowbuf + (size_t)(k & 1) * D : K;  // row k before its update
+            // ---- w of step k - 1 and x = row k of A^(k) (v_{k-1}[k] = 1) ----
+#pragma unroll
+            for (int u = U0; u < E; ++u) {
+                const int j = tid + TS_T * u;
+                const bool in = j >= k && j < D;
+                x[u] = in ? __ldcg(rb + j) : 0.0;
+                w[u] = in && k ? __ldcg(pb + j) : 0.0;
             }
-            if (tid == 0) s_b[0] = wp[k];
-            pv = ts_block_sum(pv, red, 0);
-        }
-        const double gam = 0.5 * t * pv, wk = k ? s_b[0] - gam : 0.0;
-        double s = 0.0;
-        for (int j = k + tid; j < D; j += TS_T) {
-            double x = __ldcg(rb + j);
             if (k) {
-                const double v = vp[j], w = fma(-gam, v, wp[j]);
-                wp[j] = w;
-                x = fma(-wk, v, x - w);
-            }
-            vc[j] = x;
-            if (j >= k + 2) s = fma(x, x, s);
-            if (j == k + 1) s_b[1] = x;
-            if (j == k && c == 0) dg[k] = x;
-        }
-        const double xn2 = ts_block_sum(s, red, 1), x0 = s_b[1];
-        double beta = x0, scal = 0.0;
-        t = 0.0;
-        if (xn2 > 0.0) {
-            const double S = fma(x0, x0, xn2);
-            if (S > 1e-290 && S < 1e290) {
-                const double y = fast_rsqrt(S);
-                double b = S * y;
-                b = fma(0.5 * fma(-b, b, S), y, b);
-                t = fma(fabs(x0), y, 1.0);  // (beta - x0) / beta with beta = -sign(x0) sqrt(S)
-                beta = -copysign(b, x0);
-                scal = copysign(fast_rcp(fabs(x0) + b), x0);
-            } else {
-                beta = -copysign(sqrt(S), x0);
-                t = (beta - x0) / beta;
-                scal = 1.0 / (x0 - beta);
-            }
-        }
-        for (int j = k + 1 + tid; j < D; j += TS_T) {
-            const double v = j == k + 1 ? 1.0 : vc[j] * scal;
-            vc[j] = v;
-            if (c == 0) Hv[(int64_t)k * D + j] = v;
-        }
-        if (c == 0 && tid == 0) {
-            tau[k] = t;
-            ofd[k] = beta;
-        }
-        __syncthreads();
-        // ---- own rows i > k: the pending update, then p_i = t (row_i . v_k) ----
-        const int l0 = k >= c ? (k - c) / G + 1 : 0;
-        for (int lc = l0; lc < nl; lc += 4) {
-            double acc[4] = {}, vi[4], wi[4];
-            const int nr = min(4, nl - lc);
+                double pv = 0.0;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int i = c + (lc + (u < nr ? u : 0)) * G;
-                vi[u] = vp[i];
-                wi[u] = wp[i];
-            }
-            const bool pub = c + lc * G == k + 1;  // the next pivot row is always the first one left
-            for (int j = k + 1 + tid; j < D; j += TS_T) {
-                const double wj = wp[j], vj = vp[j], bj = vc[j];
+                for (int u = U0; u < E; ++u) pv = fma(w[u], vp[u], pv);
+                if (tid + TS_T * U0 == k) s_b[0] = w[U0];
+                pv = ts_block_sum(pv, red, 0);
+                const double gam = 0.5 * t * pv, wk = s_b[0] - gam;
 #pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    if (u < nr) {
-                        double *const ar = A + (size_t)(lc + u) * D + j;
-                        double a = *ar;
-                        if (k) {
-                            a = fma(-vi[u], wj, a);
-                            a = fma(-wi[u], vj, a);
-                            *ar = a;
-                        }
-                        if (u == 0 && pub) __stcg(rowbuf + (size_t)((k + 1) & 1) * D + j, a);
-                        acc[u] = fma(a, bj, acc[u]);
+                for (int u = U0; u < E; ++u) {
+                    w[u] = fma(-gam, vp[u], w[u]);
+                    x[u] = fma(-wk, vp[u], x[u] - w[u]);
+                }
+            }
+            double s = 0.0;
+#pragma unroll
+            for (int u = U0; u < E; ++u) {
+                const int j = tid + TS_T * u;
+                const double y = u > U0 + 1 || j >= k + 2 ? x[u] : 0.0;
+                s = fma(y, y, s);
+                if (j == k + 1) s_b[1] = x[u];
+            }
+            if (tid + TS_T * U0 == k && c == 0) dg[k] = x[U0];
+            const double xn2 = ts_block_sum(s, red, 1), x0 = s_b[1];
+            double beta = x0, scal = 0.0;
+            t = 0.0;
+            if (xn2 > 0.0) {
+                const double S = fma(x0, x0, xn2);
+                if (S > 1e-290 && S < 1e290) {
+                    const double y = fast_rsqrt(S), b = S * y;
+                    t = fma(fabs(x0), y, 1.0);  // (beta - x0) / beta with beta = -sign(x0) sqrt(S)
+                    beta = -copysign(b, x0);
+                    scal = copysign(fast_rcp(fabs(x0) + b), x0);
+                } else {
+                    beta = -copysign(sqrt(S), x0);
+                    t = (beta - x0) / beta;
+                    scal = 1.0 / (x0 - beta);
+                }
+            }
+#pragma unroll
+            for (int u = U0; u < E; ++u) {
+                const int j = tid + TS_T * u;
+                vc[u] = x[u] * scal;
+                if (u <= U0 + 1) vc[u] = j == k + 1 ? 1.0 : j > k ? vc[u] : 0.0;
+                if (j > k && j < D) {
+                    vc_s[j] = vc[u];
+                    w_s[j] = w[u];
+                    if (c == 0) Hv[(int64_t)k * D + j] = vc[u];
+                }
+            }
+            if (c == 0 && tid == 0) {
+                tau[k] = t;
+                ofd[k] = beta;
+            }
+            __syncthreads();
+            // ---- own rows i > k: the pending update, then p_i = t (row_i . v_k); NR rows at a time ----
+            const int l0 = k >= c ? (k - c) / G + 1 : 0;
+            auto pass = [&](auto nrc, int lc) {
+                constexpr int NR = decltype(nrc)::value;
+                double acc[4] = {}, vi[NR], wi[NR];
+#pragma unroll
+                for (int r = 0; r < NR; ++r) {
+                    vi[r] = vp_s[c + (lc + r) * G];
+                    wi[r] = w_s[c + (lc + r) * G];
+                }
+                const bool pub = c + lc * G == k + 1;  // the next pivot row is always the first one left
+                double *const base = A + (size_t)lc * D + tid;
+                double *const prow = rowbuf + (size_t)((k + 1) & 1) * D + tid;
+#pragma unroll
+                for (int u = U0; u < E; ++u) {
+                    const bool in = tid + TS_T * u < D;
+                    double a[NR];
+#pragma unroll
+                    for (int r = 0; r < NR; ++r) a[r] = in ? base[(size_t)r * D + TS_T * u] : 0.0;
+#pragma unroll
+                    for (int r = 0; r < NR; ++r) {
+                        a[r] = fma(-vi[r], w[u], a[r]);
+                        a[r] = fma(-wi[r], vp[u], a[r]);
+                        acc[r] = fma(a[r], vc[u], acc[r]);
+                        if (in) base[(size_t)r * D + TS_T * u] = a[r];
                     }
-            }
-            // lane's row: 2 (bit 4) + (bit 3)
-            const bool h4 = lane & 16, h3 = lane & 8;
-            const double a0 = (h4 ? acc[2] : acc[0]) + __shfl_xor_sync(FULL, h4 ? acc[0] : acc[2], 16);
-            const double a1 = (h4 ? acc[3] : acc[1]) + __shfl_xor_sync(FULL, h4 ? acc[1] : acc[3], 16);
-            double x = (h3 ? a1 : a0) + __shfl_xor_sync(FULL, h3 ? a0 : a1, 8);
+                    if (pub && in) __stcg(prow + TS_T * u, a[0]);
+                }
+                // sums over the warp: with four rows lane's row is 2 (bit 4) + (bit 3), with two bit 4
+                const bool h4 = lane & 16, h3 = lane & 8;
+                double y;
+                int row = 0;
+                if constexpr (NR == 4) {
+                    const double a0 = (h4 ? acc[2] : acc[0]) + __shfl_xor_sync(FULL, h4 ? acc[0] : acc[2], 16);
+                    const double a1 = (h4 ? acc[3] : acc[1]) + __shfl_xor_sync(FULL, h4 ? acc[1] : acc[3], 16);
+                    y = (h3 ? a1 : a0) + __shfl_xor_sync(FULL, h3 ? a0 : a1, 8);
+                    row = (h4 ? 2 : 0) + (h3 ? 1 : 0);
+                } else {
+                    if constexpr (NR == 2) {
+                        y = (h4 ? acc[1] : acc[0]) + __shfl_xor_sync(FULL, h4 ? acc[0] : acc[1], 16);
+                        row = h4 ? 1 : 0;
+                    } else {
+                        y = acc[0] + __shfl_xor_sync(FULL, acc[0], 16);
+                    }
+                    y += __shfl_xor_sync(FULL, y, 8);
+                }
 #pragma unroll
-            for (int o = 4; o; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
-            if ((lane & 7) == 0 && (lane >> 3) < nr) part[wid * maxl + lc + (lane >> 3)] = x;
+                for (int o = 4; o; o >>= 1) y += __shfl_xor_sync(FULL, y, o);
+                if ((lane & (NR == 4 ? 7 : NR == 2 ? 15 : 31)) == 0) part[wid * maxl + lc + row] = y;
+            };
+            int lc = l0;
+            for (; lc + 4 <= nl; lc += 4) pass(std::integral_constant<int, 4>(), lc);
+            if (lc + 2 <= nl) {
+                pass(std::integral_constant<int, 2>(), lc);
+                lc += 2;
+            }
+            if (lc < nl) pass(std::integral_constant<int, 1>(), lc);
+            __syncthreads();
+            for (int l = l0 + tid; l < nl; l += TS_T)
+                __stcg(pbuf + (size_t)(k & 1) * D + c + l * G,
+                       t * ((part[l] + part[maxl + l]) + (part[2 * maxl + l] + part[3 * maxl + l])));
+            if (!grid_barrier_spin(bar_count, target)) {
+                if (tid == 0) atomicOr(status, ST_TIMEOUT);
+                alive = false;  // the whole block
+            }
+            // v_k becomes v_{k-1}
+            double *const o = vp_s;
+            vp_s = vc_s;
+            vc_s = o;
+#pragma unroll
+            for (int u = U0; u < E; ++u) vp[u] = vc[u];
         }
-        __syncthreads();
-        for (int l = l0 + tid; l < nl; l += TS_T)
-            __stcg(pbuf + (size_t)(k & 1) * D + c + l * G,
-                   t * ((part[l] + part[maxl + l]) + (part[2 * maxl + l] + part[3 * maxl + l])));
-        if (!grid_barrier_spin(bar_count, target)) {
-            if (tid == 0) atomicOr(status, ST_TIMEOUT);
-            return;
-        }
-        double *const o = vp;  // v_k becomes v_{k-1}
-        vp = vc;
-        vc = o;
-    }
+    });
+    if (!alive) return;
     // the last 2 x 2 block: row a from its owner's published copy, the corner from the owner itself
     const int a = D - 2, b = D - 1, k = D - 2;
     const double *const pb = pbuf + (size_t)((k & 1) ^ 1) * D, *const rb = rowbuf + (size_t)(k & 1) * D;
     if (tid == 0) {
-        const double pa = __ldcg(pb + a), pbb = __ldcg(pb + b), pv = fma(pa, vp[a], pbb * vp[b]);
-        const double gam = 0.5 * t * pv, wa = fma(-gam, vp[a], pa), wb = fma(-gam, vp[b], pbb);
+        const double va = vp_s[a], vb = vp_s[b], pa = __ldcg(pb + a), pbb = __ldcg(pb + b), pv = fma(pa, va, pbb * vb);
+        const double gam = 0.5 * t * pv, wa = fma(-gam, va, pa), wb = fma(-gam, vb, pbb);
         if (c == 0) {
-            dg[a] = __ldcg(rb + a) - 2.0 * vp[a] * wa;
-            ofd[a] = __ldcg(rb + b) - vp[a] * wb - wa * vp[b];
+            dg[a] = __ldcg(rb + a) - 2.0 * va * wa;
+            ofd[a] = __ldcg(rb + b) - va * wb - wa * vb;
             tau[a] = 0.0;
         }
-        if (b % G == c) dg[b] = A[(size_t)(b / G) * D + b] - 2.0 * vp[b] * wb;
+        if (b % G == c) dg[b] = A[(size_t)(b / G) * D + b] - 2.0 * vb * wb;
     }
 }
 
@@ -388,7 +444,7 @@ __device__ __forceinline__ int sturm_below_f(const float *dg, const float *e2, i
 // "at least i + 1 eigenvalues at or above".  float32 rounds narrow the interval to about 1e-5 ||T|| first
 // (a float32 count takes a seventh of the time); the first FP64 round then checks both its ends and
 // falls back to the Gershgorin interval's part beyond an end that does not hold.
-// 160 eigenvalues of D = 768: 4.93 ms with 31 points, FP64 throughout and a division a pivot; @@ now.
+// 160 eigenvalues of D = 768: 4.93 ms with 31 points, FP64 throughout and a division a pivot; 1.31 ms now.
 __global__ void __launch_bounds__(64) bisect_kernel(const double *dg, const double *ofd, int D, int nout, double lo0,
                                                     double hi0, double pivmin, double *lam) {
     extern __shared__ double sb[];
@@ -468,9 +524,10 @@ __device__ __forceinline__ double start_entry(int i, int e) {
 // against the cluster's earlier vectors (modified Gram-Schmidt), normalise -- three rounds (the
 // eigenvalue is accurate to the last bits, so one solve already nearly converges).  Z: nout x D.
 // The factors and the vector sit in shared memory and the recurrences in registers, so that a chain step
-// costs its FP64 instructions alone: 160 vectors of D = 768 1.15 ms with the factors in L2 and two
-// divisions a row, @@ now.
-__global__ void __launch_bounds__(128) inviter_kernel(const double *dg, const double *ofd, int D, const double *lam,
+// costs its FP64 instructions alone; three warps a block, so that the chains of two blocks on an SM
+// fall on different schedulers: 160 vectors of D = 768 1.15 ms with the factors in L2 and two
+// divisions a row, 0.69 ms now.
+__global__ void __launch_bounds__(96) inviter_kernel(const double *dg, const double *ofd, int D, const double *lam,
                                                       const int *cb, const int *ce, double tol, double *Z) {
     extern __shared__ double si[];
     __shared__ double red[4];
@@ -562,57 +619,71 @@ __global__ void __launch_bounds__(128) inviter_kernel(const double *dg, const do
     }
 }
 
+template <int T>
+__device__ __forceinline__ double bt_block_sum(double x, double (*red)[T / 32], int slot) {
+    x = warp_sum_d(x);
+    if ((threadIdx.x & 31) == 0) red[slot][threadIdx.x >> 5] = x;
+    __syncthreads();
+    double s = red[slot][0];
+#pragma unroll
+    for (int w = 1; w < T / 32; ++w) s += red[slot][w];
+    return s;
+}
+
 // evecs[r] = Q z_r = H_0 H_1 .. H_{D-3} z_r, unit norm, largest-magnitude entry positive (first
-// index on ties); evals[r] = lam[r] (evals nullable).  One block of four warps per eigenvector, its
-// entries in registers (tid + 128 u), the next reflection's vector loaded while the current one's sum
-// goes round: 160 vectors of D = 768 2.04 ms with one warp per vector, @@ now.
-template <int E>
-__global__ void __launch_bounds__(TS_T) backtrans_kernel(const double *__restrict__ Z, const double *__restrict__ Hv,
+// index on ties); evals[r] = lam[r] (evals nullable).  One block of T threads per eigenvector, its
+// entries in registers (tid + T u), the next reflection's vector loaded while the current one's sum goes
+// round: 160 vectors of D = 768 2.04 ms with one warp per vector, 1.12 ms with the slots below the
+// reflection predicated off instead of left out, 0.87 ms now.
+template <int T, int E>
+__global__ void __launch_bounds__(T) backtrans_kernel(const double *__restrict__ Z, const double *__restrict__ Hv,
                                                          const double *__restrict__ tau, int D, const double *lam,
                                                          double *evals, double *evecs) {
-    __shared__ double red[2][TS_W];
-    __shared__ double s_best[TS_W];
-    __shared__ int s_bi[TS_W];
+    __shared__ double red[2][(T / 32)];
+    __shared__ double s_best[(T / 32)];
+    __shared__ int s_bi[(T / 32)];
     const int r = blockIdx.x, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     double x[E], v[E];
 #pragma unroll
-    for (int u = 0; u < E; ++u) x[u] = tid + TS_T * u < D ? Z[(size_t)r * D + tid + TS_T * u] : 0.0;
+    for (int u = 0; u < E; ++u) x[u] = tid + T * u < D ? Z[(size_t)r * D + tid + T * u] : 0.0;
     auto fetch = [&](int k) {
 #pragma unroll
         for (int u = 0; u < E; ++u) {
-            const int j = tid + TS_T * u;
+            const int j = tid + T * u;
             v[u] = k >= 0 && j > k && j < D ? __ldg(Hv + (int64_t)k * D + j) : 0.0;
         }
     };
     fetch(D - 3);
-    for (int k = D - 3; k >= 0; --k) {
-        const int u0 = (k + 1) / TS_T;  // entries below 128 u0 are zero in v
-        double w[E], s = 0.0;
+    // phase U0, from the last: the reflections k with (k + 1) / T = U0, whose entries sit in slots U0 ..
+    phases(std::integral_constant<int, E>(), [&](auto ic) {
+        constexpr int U0 = E - 1 - decltype(ic)::value;
+        for (int k = min(D - 3, T * (U0 + 1) - 2); k >= max(0, T * U0 - 1); --k) {
+            double w[E], s = 0.0;
 #pragma unroll
-        for (int u = 0; u < E; ++u) {
-            w[u] = v[u];
-            if (u >= u0) s = fma(w[u], x[u], s);
+            for (int u = U0; u < E; ++u) {
+                w[u] = v[u];
+                s = fma(w[u], x[u], s);
+            }
+            const double t = __ldg(tau + k);
+            fetch(k - 1);
+            s = -bt_block_sum<T>(s, red, k & 1) * t;
+#pragma unroll
+            for (int u = U0; u < E; ++u) x[u] = fma(s, w[u], x[u]);
         }
-        const double t = __ldg(tau + k);
-        fetch(k - 1);
-        s = -ts_block_sum(s, red, k & 1) * t;
-#pragma unroll
-        for (int u = 0; u < E; ++u)
-            if (u >= u0) x[u] = fma(s, w[u], x[u]);
-    }
+    });
     double s = 0.0, best = -1.0;
     int bi = D;
 #pragma unroll
     for (int u = 0; u < E; ++u) {
         s = fma(x[u], x[u], s);
         const double a = fabs(x[u]);
-        if (tid + TS_T * u < D && a > best) {
+        if (tid + T * u < D && a > best) {
             best = a;
-            bi = tid + TS_T * u;
+            bi = tid + T * u;
         }
     }
     __syncthreads();
-    s = ts_block_sum(s, red, 0);
+    s = bt_block_sum<T>(s, red, 0);
     // largest |x_i|, first index on ties
 #pragma unroll
     for (int o = 16; o; o >>= 1) {
@@ -628,7 +699,7 @@ __global__ void __launch_bounds__(TS_T) backtrans_kernel(const double *__restric
         s_bi[wid] = bi;
     }
     __syncthreads();
-    for (int w = 0; w < TS_W; ++w)
+    for (int w = 0; w < (T / 32); ++w)
         if (s_best[w] > best || (s_best[w] == best && s_bi[w] < bi)) {
             best = s_best[w];
             bi = s_bi[w];
@@ -636,28 +707,28 @@ __global__ void __launch_bounds__(TS_T) backtrans_kernel(const double *__restric
     __shared__ double s_sign;
 #pragma unroll
     for (int u = 0; u < E; ++u)
-        if (tid + TS_T * u == bi) s_sign = x[u] < 0.0 ? -1.0 : 1.0;
+        if (tid + T * u == bi) s_sign = x[u] < 0.0 ? -1.0 : 1.0;
     __syncthreads();
     const double scale = (s > 0.0 ? 1.0 / sqrt(s) : 0.0) * (bi < D ? s_sign : 1.0);
 #pragma unroll
     for (int u = 0; u < E; ++u)
-        if (tid + TS_T * u < D) evecs[(size_t)r * D + tid + TS_T * u] = x[u] * scale;
+        if (tid + T * u < D) evecs[(size_t)r * D + tid + T * u] = x[u] * scale;
     if (tid == 0 && evals) evals[r] = lam[r];
 }
 
 static int launch_backtrans(const double *Z, const double *Hv, const double *tau, int D, int nout, const double *lam,
                             double *evals, double *evecs, cudaStream_t st) {
-    auto go = [&](auto k) -> int {
-        k<<<nout, TS_T, 0, st>>>(Z, Hv, tau, D, lam, evals, evecs);
+    auto go = [&](auto k, int threads) -> int {
+        k<<<nout, threads, 0, st>>>(Z, Hv, tau, D, lam, evals, evecs);
         LV_CHECK_LAUNCH("backtrans_kernel");
         return LV_OK;
     };
-    if (D <= 2 * TS_T) return go(backtrans_kernel<2>);
-    if (D <= 4 * TS_T) return go(backtrans_kernel<4>);
-    if (D <= 6 * TS_T) return go(backtrans_kernel<6>);
-    if (D <= 8 * TS_T) return go(backtrans_kernel<8>);
-    if (D <= 16 * TS_T) return go(backtrans_kernel<16>);
-    return go(backtrans_kernel<32>);
+    if (D <= 256) return go(backtrans_kernel<128, 2>, 128);
+    if (D <= 512) return go(backtrans_kernel<128, 4>, 128);
+    if (D <= 768) return go(backtrans_kernel<128, 6>, 128);
+    if (D <= 1024) return go(backtrans_kernel<128, 8>, 128);
+    if (D <= 2048) return go(backtrans_kernel<128, 16>, 128);
+    return go(backtrans_kernel<128, 32>, 128);
 }
 
 // the path applies: 8 <= D <= 4096, 1 <= nout <= D
@@ -679,7 +750,7 @@ int eigh_top(const double *K, int D, int nout, double *evals, double *evecs, cud
     // rows in shared memory while they fit (D <= about 1800); two rows a block at least
     const int gs = std::min(sms, (D + 1) / 2), maxl = (D + gs - 1) / gs;
     const size_t ssm = sizeof(double) * ((size_t)maxl * D + 3 * (size_t)D + (size_t)TS_W * maxl);
-    const bool in_sm = ssm <= 220 * 1024;
+    const bool in_sm = ssm <= 220 * 1024 && D <= 16 * TS_T;
     const size_t tsm = sizeof(double) * (3 * (size_t)D + TRI_WARPS);
     const size_t bsm = 2 * sizeof(double) * (size_t)D + 2 * sizeof(float) * (size_t)D, ism = (5 * sizeof(double) + 1) * (size_t)D;
     if ((!in_sm && tmp_alloc((void **)&A, sizeof(double) * DD, st)) || tmp_alloc((void **)&Hv, sizeof(double) * DD, st) ||
@@ -699,7 +770,12 @@ int eigh_top(const double *K, int D, int nout, double *evals, double *evecs, cud
     }
     // 1. tridiagonal form: one block per SM, all co-resident (cooperative launch)
     {
-        const void *kern = in_sm ? (const void *)tridiag_sm_kernel : (const void *)tridiag_kernel;
+        const void *kern = !in_sm            ? (const void *)tridiag_kernel
+                           : D <= 2 * TS_T  ? (const void *)tridiag_sm_kernel<2>
+                           : D <= 4 * TS_T  ? (const void *)tridiag_sm_kernel<4>
+                           : D <= 6 * TS_T  ? (const void *)tridiag_sm_kernel<6>
+                           : D <= 8 * TS_T  ? (const void *)tridiag_sm_kernel<8>
+                                            : (const void *)tridiag_sm_kernel<16>;
         const size_t sm = in_sm ? ssm : tsm;
         const int threads = in_sm ? TS_T : TRI_THREADS, blocks = in_sm ? gs : sms;
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess ||
@@ -776,7 +852,7 @@ int eigh_top(const double *K, int D, int nout, double *evals, double *evecs, cud
             goto done;
         }
         const double tol = std::max(DBL_EPSILON * tnorm, DBL_MIN);
-        inviter_kernel<<<nclus, 128, ism, st>>>(dg, ofd, D, lam, cl, cl + nclus, tol, Z);
+        inviter_kernel<<<nclus, 96, ism, st>>>(dg, ofd, D, lam, cl, cl + nclus, tol, Z);
         if (cudaGetLastError() != cudaSuccess) {
             rc = fail(LV_ERR_CUDA, "eigh_top: inverse iteration launch failed");
             goto done;
