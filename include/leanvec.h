@@ -399,7 +399,10 @@ typedef struct {
                                 max(1024, 4 L) up to 8192 slots of 32-bit ids; twice as many 16-bit
                                 tags with visited_bits 16; with visited_bits 0 as well, 2048 or 1024
                                 tags for long walks, see visited_bits) */
-    int32_t warps_per_block; /* 0 = default */
+    int32_t warps_per_block; /* 0 = default.  When this, warps_per_query, queries_per_warp, hash_slots and
+                                visited_bits are all 0, stats is NULL, the primaries are LVQ records
+                                and width <= 2, a batch of at most 6 queries per SM is searched with
+                                a block of four warps per query (same results, shorter walks) */
     int32_t width;           /* search width: beam members expanded per round, 1..4 (0 = 1);
                                 width * R <= 256.  1 is the classic best-first traversal */
     int32_t warps_per_query; /* warps that serve one query, 1, 2 or 4, dividing width (0 = 1):

@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "beam.cuh"
+#include "beam_block.cuh"
 #include "common.cuh"
 #include "index.cuh"
 
@@ -99,6 +100,12 @@ int ensure_ws(void **p, size_t *have, size_t want) {
 int *index_status(lv_index *idx) { return idx->status; }
 int index_num_sms(lv_index *idx) { return idx->num_sms; }
 
+// Queries per SM up to which a batch runs with a block per query.  Time of a warp per query over that of a
+// block (200k x 768, L = 128 / 1M x 200, L = 300 / L2 200k x 960, L = 72 / 10k x 128, L = 50): 100 queries 1.15 /
+// 1.33 / 1.30 / 1.11, 608 1.20 / 1.37 / 1.27 / 1.09, 912 (six per SM) 1.07 / 1.20 / 1.23 / 1.06, 1216 0.82 /
+// 0.86 / 1.13 / 1.01, 1520 0.83 / 0.87 / 0.84 / 0.97.
+constexpr int BLOCK_QUERIES = 6;
+
 static int next_pow2(int x) {
     int p = 1;
     while (p < x) p <<= 1;
@@ -184,12 +191,29 @@ int search_shape(const lv_index *idx, const lv_search_params *params, BeamParams
     }
     if (*smem > 227 * 1024) return fail(LV_ERR_CAPACITY, w + ": L / hash_slots too large for shared memory");
     *block = warps * 32;
+    // Small batches, where the caller leaves the launch shape open: a block per query.  (Calls that ask for
+    // the counters keep a warp per query: `scored` counts what that shape's cache forgets, and is the
+    // same for a batch and for its parts.)
+    const bool open = params->warps_per_block <= 0 && params->warps_per_query <= 0 && qpw == 0 && vb == 0 &&
+                      params->hash_slots <= 0;
+    if (open && !p.stats && idx->pbits != 32 && p.W <= 2 && p.m <= (int64_t)BLOCK_QUERIES * idx->num_sms) {
+        p.qpw = 0;
+        p.vbits = 32;
+        p.Hcap = 4096;
+        p.hbits = 12;  // log2(4096)
+        p.Rcap = (int)round_up(p.W * idx->R, 32);
+        p.warp_smem = block_query_smem(p.Lcap, p.Hcap, p.Rcap, qbytes);
+        *smem = (size_t)p.warp_smem;
+        *block = BB_T;
+    }
     return LV_OK;
 }
 
 int launch_beam_search(const lv_index *idx, const BeamParams &p, int block, size_t smem, cudaStream_t st) {
     if (idx->pbits == 32) return launch_search_fp32(p, (idx->pg.code_chunks + 31) / 32, block, smem, idx->num_sms, st);
     const int nc = (idx->pg.code_chunks + 1 + idx->metric + 3) / 4;  // codes + constants chunks over 4 lanes
+    if (p.qpw == 0)
+        return idx->pbits == 8 ? launch_search_block8(p, nc, smem, st) : launch_search_block4(p, nc, smem, st);
     if (p.qpw == 2)
         return idx->pbits == 8 ? launch_search_half8(p, nc, block, smem, idx->num_sms, st)
                                : launch_search_half4(p, nc, block, smem, idx->num_sms, st);

@@ -73,7 +73,8 @@ struct BeamParams {
     int W;      // search width: parents expanded per round (1..4, W * R <= 256)
     int T;      // warps per query (1, 2 or 4; divides W); Rcap = T * (W / T * R rounded up to 32)
     int warp_smem;  // shared bytes of one query (one team of T warps, or one half warp)
-    int qpw;        // queries per warp: 1 (beam_kernel) or 2 (beam_half_kernel, beam_half.cuh)
+    int qpw;        // queries per warp: 1 (beam_kernel) or 2 (beam_half_kernel, beam_half.cuh); 0: a block
+                    // per query (beam_block_kernel, beam_block.cuh)
     int64_t *slots;  // host side: when set, the search launchers report the query slots one
                      // launch keeps resident (blocks per SM x SMs x teams per block) and launch nothing
 };
@@ -1067,6 +1068,9 @@ int launch_search_fp32_tags(const BeamParams &p, int ncw, int block, size_t smem
 // two queries per warp: LVQ-8 primaries with nc = 1..4 chunks per lane, LVQ-4 with 1..3
 int launch_search_half8(const BeamParams &p, int nc, int block, size_t smem, int num_sms, cudaStream_t st);
 int launch_search_half4(const BeamParams &p, int nc, int block, size_t smem, int num_sms, cudaStream_t st);
+// a block per query (small batches): LVQ-8 primaries with nc = 1..4 chunks per lane, LVQ-4 with 1..3
+int launch_search_block8(const BeamParams &p, int nc, size_t smem, cudaStream_t st);
+int launch_search_block4(const BeamParams &p, int nc, size_t smem, cudaStream_t st);
 int launch_build_search(const BeamParams &p, int bits, int nc, int block, size_t smem, int num_sms,
                         cudaStream_t st);
 // scores the candidates the RERANK beam kernel handed over (p.cand, p.cand_n) and writes p.ids / p.scores
