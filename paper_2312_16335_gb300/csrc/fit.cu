@@ -279,20 +279,22 @@ __global__ void f64_to_f32_kernel(const double *__restrict__ a, int64_t n, float
 
 // ------------------------------------------------- Jacobi eigh of small matrices
 // The whole decomposition of a matrix of up to JC_MAX rows in one launch: a cluster of JC_CL blocks
-// keeps A in its shared memory (row i in block i mod JC_CL, entries j >= i; two copies, one read and
+// keeps A in its shared memory (row i in block i mod JC_CL, entries j > i; two copies, one read and
 // one written in turn) and goes from round to round over the cluster barrier.  A round on the
 // pairs (p_k, q_k) splits A into 2 x 2 blocks (pair I x pair J), each owned by one thread, which reads it
-// from the old copy, applies both rotations and writes it to the new one; every block forms all
-// rotations itself.  The rotations are kept, and jacobi_vectors_kernel applies them to the rows of V,
-// which do not depend on one another, over all SMs.
+// from the old copy, applies both rotations and writes it to the new one.  Every block forms all
+// rotations itself from copies of its own: the diagonal, which it updates for itself, and the
+// round's a_pq, which their owners send to all blocks as they write them.  The rotations are kept, and
+// jacobi_vectors_kernel applies them to the rows of V, which do not depend on one another, over all SMs.
 //
 // FP64 bounds this: the pipe takes a warp instruction every 64 cycles, so a division or a root
 // costs 550 and no extra warp hides it.  Hence the angle comes from float32 (any t serves that
-// brings a_pq down -- 1e-7 of it remains, the next sweep's share), and only c = 1 / sqrt(1 + t^2) and
-// s = t c are made accurate to FP64: a float32 rsqrt with one cubic step.  The update multiplies by t
-// and scales by c_I c_J at the end (12 instead of 16 operations).
+// brings a_pq down -- 1e-7 of it remains, the next sweep's share), converted by integer instructions, and
+// only c = 1 / sqrt(1 + t^2) and s = t c are made accurate to FP64: an approximate root with one cubic
+// step.  The update multiplies by t and scales by c_I c_J at the end (12 instead of 16 operations).
 // 128 rows, 7 sweeps of 127 rounds: 5.4 ms of kernels and 2 ms of graph building with two launches a
-// round replayed from a graph made per call, 2.7 ms and 0.2 ms for the vectors now.
+// round replayed from a graph made per call; 2.7 ms with the angles' entries read from the other
+// blocks in every round; 1.9 ms now, and 0.2 ms for the vectors.
 constexpr int JC_CL = 16, JC_MAX = 256, JC_SWEEPS = 40;
 
 __device__ __forceinline__ double ld_cluster(uint32_t addr, int rank) {
@@ -311,23 +313,32 @@ __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
+// v 2^-e as float32 (truncated; 0 below its range), e an exponent field >= v's: integer instructions only
+__device__ __forceinline__ float scaled_float(double v, int e) {
+    const int hi = __double2hiint(v), x = ((hi >> 20) & 0x7ff) - e + 127;
+    const unsigned m = ((unsigned)hi & 0xfffffu) << 3 | (unsigned)__double2loint(v) >> 29;
+    return x > 0 ? __uint_as_float(((unsigned)hi & 0x80000000u) | (unsigned)x << 23 | m) : 0.f;
+}
+// a float32 as FP64 (0 below its normal range), integer instructions only
+__device__ __forceinline__ double float_bits_to_double(float f) {
+    const unsigned u = __float_as_uint(f), x = (u >> 23) & 0xffu;
+    if (x == 0u) return 0.0;
+    return __hiloint2double((int)((u & 0x80000000u) | (x + 896u) << 20 | (u & 0x7fffffu) >> 3), (int)(u << 29));
+}
+
 // tangent t and cosine c of the rotation that (nearly) zeroes a_pq: rows p <- c (p - t q), q <- c (q + t p)
 __device__ __forceinline__ void jacobi_angle(double app, double aqq, double apq, double &t, double &c) {
-    t = 0.0;
-    c = 1.0;
-    if (!(fabs(apq) > 1e-300)) return;
-    const double d = aqq - app, x2 = apq + apq;
-    // scaled by a power of two to fit float32
-    const int ed = __double2hiint(d) & 0x7ff00000, ex = __double2hiint(x2) & 0x7ff00000;
-    const int e = min(max(max(ed, ex), 0x00100000), 0x7fd00000);
-    const double sc = __hiloint2double(0x7fe00000 - e, 0);
-    const float theta = __double2float_rn(d * sc) / __double2float_rn(x2 * sc);
+    const double d = aqq - app;
+    const int ed = (__double2hiint(d) >> 20) & 0x7ff, ex = (__double2hiint(apq) >> 20) & 0x7ff;
+    const int e = max(ed, ex);
+    const float theta = 0.5f * scaled_float(d, e) / scaled_float(apq, e);
     const float tf = copysignf(1.0f / (fabsf(theta) + sqrtf(fmaf(theta, theta, 1.0f))), theta);
-    if (!(fabsf(tf) <= 1.0f)) return;  // 0 / 0
-    t = (double)tf;
+    // no rotation for 0 / 0, a_pq below 2^-996 (about 1e-300) or entries that are not finite
+    t = fabsf(tf) <= 1.0f && ex > 27 && e < 0x7ff ? float_bits_to_double(tf) : 0.0;
     const double u = fma(t, t, 1.0);
-    const double y = (double)rsqrtf(fmaf(tf, tf, 1.0f));
-    const double r = fma(-u, y * y, 1.0);  // about 2^-23: y (1 + r / 2 + 3 r^2 / 8) is good to r^3
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(u));  // about 2^-20
+    const double r = fma(-u, y * y, 1.0);                     // y (1 + r / 2 + 3 r^2 / 8) is good to r^3
     c = fma(y * r, fma(0.375, r, 0.5), y);
 }
 
@@ -345,11 +356,12 @@ __device__ __forceinline__ void rr_pair_fast(int r, int k, int Dp, int &p, int &
     q = max(a, b);
 }
 
-// T threads; NB: 2 x 2 blocks of a thread at most
+// T threads (h = Dp / 2 <= T / 2); NB: 2 x 2 blocks of a thread at most
 template <int T, int NB>
 __global__ void __launch_bounds__(T) jacobi_cluster_kernel(double *__restrict__ A, int Dp, double2 *__restrict__ rot,
                                                            int *__restrict__ sweeps) {
     extern __shared__ double sm_a[];
+    __shared__ double s_dg[2][JC_MAX], s_apq[2][JC_MAX / 2];
     __shared__ double2 s_tc[JC_MAX / 2];
     __shared__ double s_red[T / 32][2], s_part[2];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -358,14 +370,19 @@ __global__ void __launch_bounds__(T) jacobi_cluster_kernel(double *__restrict__ 
     const int rank = (int)crank, h = Dp / 2, rows = (Dp + JC_CL - 1) / JC_CL, rounds = Dp - 1;
     const uint32_t base = (uint32_t)__cvta_generic_to_shared(sm_a);
     const uint32_t part = (uint32_t)__cvta_generic_to_shared(s_part);
-    auto at = [&](int buf, int i, int j) {  // i <= j
-        return base + 8u * (uint32_t)((buf * rows + (i >> 4)) * Dp + j);
-    };
+    const uint32_t apq_a = (uint32_t)__cvta_generic_to_shared(&s_apq[0][0]);
+    auto at = [&](int i, int j) { return base + 8u * (uint32_t)((i >> 4) * Dp + j); };  // i < j
     static_assert(JC_CL == 16, "row to block by shifts");
     for (int l = wid; l < rows; l += T / 32) {
         const int i = rank + JC_CL * l;
         if (i < Dp)
             for (int j = i + lane; j < Dp; j += 32) sm_a[l * Dp + j] = A[(int64_t)i * Dp + j];
+    }
+    for (int i = tid; i < Dp; i += T) s_dg[0][i] = A[(int64_t)i * Dp + i];
+    if (tid < h) {
+        int p, q;
+        rr_pair_fast(0, tid, Dp, p, q);
+        s_apq[0][tid] = A[(int64_t)p * Dp + q];
     }
     // this thread's 2 x 2 blocks: pairs I < J of the round's list, the same positions in every round
     int bI[NB], bJ[NB];
@@ -392,14 +409,12 @@ __global__ void __launch_bounds__(T) jacobi_cluster_kernel(double *__restrict__ 
         for (int l = wid; l < rows; l += T / 32) {
             const int i = rank + JC_CL * l;
             if (i < Dp)
-                for (int j = i + lane; j < Dp; j += 32) {
+                for (int j = i + 1 + lane; j < Dp; j += 32) {
                     const double v = sm_a[(buf * rows + l) * Dp + j];
-                    if (j == i)
-                        diag = fma(v, v, diag);
-                    else
-                        off = fma(v, v, off);
+                    off = fma(v, v, off);
                 }
         }
+        for (int i = rank + JC_CL * tid; i < Dp; i += JC_CL * T) diag = fma(s_dg[buf][i], s_dg[buf][i], diag);
         for (int o = 16; o; o >>= 1) {
             off += __shfl_xor_sync(FULL, off, o);
             diag += __shfl_xor_sync(FULL, diag, o);
@@ -424,18 +439,10 @@ __global__ void __launch_bounds__(T) jacobi_cluster_kernel(double *__restrict__ 
         const double tot = off + diag;
         if (!(off > 1e-28 * tot) || tot == 0.0 || sweep == JC_SWEEPS) break;
         for (int r = 0; r < rounds; ++r, buf ^= 1) {
-            double app = 0.0, aqq = 0.0, apq = 0.0;
-            int p = 0, q = 0;
-            if (tid < h) {
-                rr_pair_fast(r, tid, Dp, p, q);
-                app = ld_cluster(at(buf, p, p), p & 15);
-                aqq = ld_cluster(at(buf, q, q), q & 15);
-                apq = ld_cluster(at(buf, p, q), p & 15);
-            }
-            // entries (p_I, p_J), (p_I, q_J), (q_I, p_J), (q_I, q_J)
+            const uint32_t from = 8u * (uint32_t)(buf * rows * Dp), to = 8u * (uint32_t)((buf ^ 1) * rows * Dp);
+            // entries (p_I, p_J), (p_I, q_J), (q_I, p_J), (q_I, q_J), on their way while the angles are formed
             double v[NB][4];
-            uint32_t ad[NB][4];
-            int rk[NB][4];
+            int ei[NB][4], ej[NB][4];
 #pragma unroll
             for (int e = 0; e < NB; ++e) {
                 if (bI[e] < 0) continue;
@@ -444,45 +451,79 @@ __global__ void __launch_bounds__(T) jacobi_cluster_kernel(double *__restrict__ 
                 rr_pair_fast(r, bJ[e], Dp, j2[0], j2[1]);
 #pragma unroll
                 for (int x = 0; x < 4; ++x) {
-                    const int i = min(i2[x >> 1], j2[x & 1]), j = max(i2[x >> 1], j2[x & 1]);
-                    ad[e][x] = at(0, i, j);
-                    rk[e][x] = i & 15;
-                    v[e][x] = ld_cluster(ad[e][x] + 8u * (uint32_t)(buf * rows * Dp), rk[e][x]);
+                    ei[e][x] = min(i2[x >> 1], j2[x & 1]);
+                    ej[e][x] = max(i2[x >> 1], j2[x & 1]);
+                    v[e][x] = ld_cluster(at(ei[e][x], ej[e][x]) + from, ei[e][x] & 15);
                 }
             }
             if (tid < h) {
+                int p, q;
+                rr_pair_fast(r, tid, Dp, p, q);
                 double t, c;
-                jacobi_angle(app, aqq, apq, t, c);
+                jacobi_angle(s_dg[buf][p], s_dg[buf][q], s_apq[buf][tid], t, c);
                 s_tc[tid] = make_double2(t, c);
-                if ((tid & 15) == rank) {  // the pair's own 2 x 2 block
-                    const double c2 = c * c, tx = t * apq;
-                    st_cluster(at(buf ^ 1, p, p), p & 15, c2 * fma(t, fma(t, aqq, -2.0 * apq), app));
-                    st_cluster(at(buf ^ 1, q, q), q & 15, c2 * fma(t, fma(t, app, 2.0 * apq), aqq));
-                    st_cluster(at(buf ^ 1, p, q), p & 15, c2 * fma(t, (app - aqq) - tx, apq));
-                    rot[((int64_t)sweep * rounds + r) * h + tid] = make_double2(c, t * c);
-                }
             }
             __syncthreads();
+            // the pairs' own 2 x 2 blocks, by the other half of the threads: the diagonal in every block's copy,
+            // what is left of a_pq and the rotation by one block
+            const int k = tid - T / 2;
+            if (k >= 0 && k < h) {
+                int p, q;
+                rr_pair_fast(r, k, Dp, p, q);
+                const double app = s_dg[buf][p], aqq = s_dg[buf][q], apq = s_apq[buf][k];
+                const double2 tc = s_tc[k];
+                const double c2 = tc.y * tc.y, x2 = apq + apq;
+                s_dg[buf ^ 1][p] = c2 * fma(tc.x, fma(tc.x, aqq, -x2), app);
+                s_dg[buf ^ 1][q] = c2 * fma(tc.x, fma(tc.x, app, x2), aqq);
+                if ((k & 15) == rank) {
+                    st_cluster(at(p, q) + to, p & 15, c2 * fma(tc.x, fma(-tc.x, apq, app - aqq), apq));
+                    rot[((int64_t)sweep * rounds + r) * h + k] = make_double2(tc.y, tc.x * tc.y);
+                }
+            }
+            const int rn = r + 1 == rounds ? 0 : r + 1;  // the next round
 #pragma unroll
             for (int e = 0; e < NB; ++e) {
-                if (bI[e] < 0) continue;
-                const double2 ti = s_tc[bI[e]], tj = s_tc[bJ[e]];
-                const double a = fma(-ti.x, v[e][2], v[e][0]), b = fma(-ti.x, v[e][3], v[e][1]);
-                const double c = fma(ti.x, v[e][0], v[e][2]), d = fma(ti.x, v[e][1], v[e][3]);
-                const double cc = ti.y * tj.y;
-                const uint32_t o = 8u * (uint32_t)((buf ^ 1) * rows * Dp);
-                st_cluster(ad[e][0] + o, rk[e][0], cc * fma(-tj.x, b, a));
-                st_cluster(ad[e][1] + o, rk[e][1], cc * fma(tj.x, a, b));
-                st_cluster(ad[e][2] + o, rk[e][2], cc * fma(-tj.x, d, c));
-                st_cluster(ad[e][3] + o, rk[e][3], cc * fma(tj.x, c, d));
+                double n[4] = {0.0, 0.0, 0.0, 0.0};
+                int nk[4] = {-1, -1, -1, -1};
+                if (bI[e] >= 0) {
+                    const double2 ti = s_tc[bI[e]], tj = s_tc[bJ[e]];
+                    const double a = fma(-ti.x, v[e][2], v[e][0]), b = fma(-ti.x, v[e][3], v[e][1]);
+                    const double c = fma(ti.x, v[e][0], v[e][2]), d = fma(ti.x, v[e][1], v[e][3]);
+                    const double cc = ti.y * tj.y;
+                    n[0] = cc * fma(-tj.x, b, a);
+                    n[1] = cc * fma(tj.x, a, b);
+                    n[2] = cc * fma(-tj.x, d, c);
+                    n[3] = cc * fma(tj.x, c, d);
+#pragma unroll
+                    for (int x = 0; x < 4; ++x) {
+                        const int i = ei[e][x], j = ej[e][x];
+                        st_cluster(at(i, j) + to, i & 15, n[x]);
+                        // the pair's position in the next round, if (i, j) is one: i + j = 2 rn mod m, or (rn, m)
+                        int u = i - rn;
+                        if (u < 0) u += rounds;
+                        int w = j - rn;
+                        if (w < 0) w += rounds;
+                        if (j == rounds ? u == 0 : u + w == rounds) nk[x] = j == rounds ? 0 : min(u, w);
+                    }
+                }
+                // the next round's a_pq to every block
+#pragma unroll
+                for (int x = 0; x < 4; ++x) {
+                    unsigned bal = __ballot_sync(FULL, nk[x] >= 0);
+                    while (bal) {
+                        const int src = __ffs(bal) - 1;
+                        bal &= bal - 1;
+                        const double y = __shfl_sync(FULL, n[x], src);
+                        const int kk = __shfl_sync(FULL, nk[x], src);
+                        if (lane < JC_CL) st_cluster(apq_a + 8u * (uint32_t)((buf ^ 1) * (JC_MAX / 2) + kk), lane, y);
+                    }
+                }
             }
             cluster_barrier();
         }
     }
-    for (int l = tid; l < rows; l += T) {
-        const int i = rank + JC_CL * l;
-        if (i < Dp) A[(int64_t)i * Dp + i] = sm_a[(buf * rows + l) * Dp + i];
-    }
+    if (rank == 0)
+        for (int i = tid; i < Dp; i += T) A[(int64_t)i * Dp + i] = s_dg[buf][i];
     if (rank == 0 && tid == 0) *sweeps = sweep;
     cluster_barrier();  // no block leaves while another may read its partial sums
 }
@@ -592,7 +633,7 @@ int eigh_impl(const double *K, int D, int nout, double *evals, double *evecs, cu
         goto done;
     }
     pad_copy_kernel<<<(unsigned)(((int64_t)Dp * Dp + 255) / 256), 256, 0, st>>>(K, D, A, V, Dp);
-    if (Dp <= JC_MAX) {
+    if (Dp >= 4 && Dp <= JC_MAX) {
         bool ran = false;
         const size_t rots = (size_t)JC_SWEEPS * (Dp - 1) * (Dp / 2);
         if (tmp_alloc((void **)&rot, sizeof(double2) * rots, st) || tmp_alloc((void **)&nsw, sizeof(int), st)) {
