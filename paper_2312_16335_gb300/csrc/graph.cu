@@ -191,7 +191,7 @@ struct PruneParams {
     const float *bscores;  // nb x Lb: the beams' build scores
     int Lb;
     int32_t *newl;         // nb x R
-    // mode 1: reverse edges; targets whose list and new sources number lo < .. <= hi
+    // mode 1: reverse edges; targets whose new sources number lo < .. <= hi
     const int64_t *offs;   // n + 1 exclusive scan (hi: sources, lo: touched count)
     const int32_t *srcs;
     const int32_t *touched;
@@ -335,13 +335,13 @@ __global__ void __launch_bounds__(NT) prune_kernel(const PruneParams pp) {
     } else {
         const int64_t o0 = pp.offs[p] >> 32, o1 = pp.offs[p + 1] >> 32;
         const int nsrc = (int)(o1 - o0);
+        if (nsrc <= pp.lo || nsrc > pp.hi) return;  // the whole block: another launch's
         // current list (compacted)
         int nl = 0;
         for (int s0 = 0; s0 < pp.R; s0 += NT) {
             const int s = s0 + tid, u = s < pp.R ? old[s] : -1;
             nl = block_append<NT>(u >= 0, u, pid, nl, pp.PMAX, s_wcnt);
         }
-        if (nl + nsrc <= pp.lo || nl + nsrc > pp.hi) return;  // the whole block: another launch's
         // the sources ascending (ranks; they are distinct), without those present
         if (nsrc > pp.PMAX && tid == 0) atomicOr(pp.status, ST_CAPACITY);
         int *const tmp = reinterpret_cast<int *>(key);  // PMAX ids by rank
@@ -781,15 +781,17 @@ int build_graph_impl(lv_index *idx, int R, int Lb, float alpha, int passes, int 
             scatter_pairs_kernel<<<(unsigned)((tp + 255) / 256), 256, 0, st>>>(newl, perm_d + b0, nb, R, offs, cnt, srcs);
             LV_CHECK_LAUNCH("reverse-edge kernels");
             const unsigned g1 = (unsigned)std::min<int64_t>(n, tp);
-            // most targets gain a few edges: pools of up to R + 32 fit many blocks on an SM; the rest
-            // (a target may receive many reverse edges in one batch) take a second launch
+            // most targets gain a few edges: the pools of those with at most 32 sources fit many blocks on an
+            // SM; the rest (a target may receive many reverse edges in one batch) take a second launch.  The
+            // line is drawn on the sources alone, which the first launch does not change: a list it rewrote
+            // must not be taken a second time
             const int small = std::min(R + 32, PMAX1);
             for (int tier = 0; tier < (small < PMAX1 ? 2 : 1) && !rc; ++tier) {
                 PruneParams pr = pp;
                 pr.PMAX = tier ? PMAX1 : small;
                 pr.slot = prune_slot(pr.PMAX, idx->pg.code_chunks, idx->metric);
-                pr.lo = tier ? small : -1;
-                pr.hi = tier || small == PMAX1 ? 0x7fffffff : small;
+                pr.lo = tier ? 32 : -1;
+                pr.hi = tier || small == PMAX1 ? 0x7fffffff : 32;
                 rc = idx->pbits == 8 ? launch_prune<8>(pr, 1, g1, st) : launch_prune<4>(pr, 1, g1, st);
             }
             if (rc) return rc;

@@ -35,3 +35,23 @@ def test_prune_edges(n, d, bits, R, Lb, alpha, batch, rule):
     g, e = idx.get_graph()
     assert e == e_ref
     np.testing.assert_array_equal(g.cpu().numpy(), g_ref)
+
+
+def test_prune_rewritten_list_once():
+    """A list that the launch for few sources made longer counts as one of few sources still: here a target
+    of 12 neighbours or so gains a list which, with its sources again, is longer than a small pool, and
+    which must not take back the sources that the pruning left out."""
+    import paper_2312_16335_gb300 as lv
+    n, d, R = 3000, 32, 48
+    rng = np.random.default_rng(n + d)
+    means = rng.standard_normal((3, d))
+    Y = workloads.unit_rows(means[rng.integers(0, 3, n)] + rng.standard_normal((n, d)))
+    mu = oracle.mean_fp32(Y)
+    kw = dict(R=R, L_build=64, alpha=0.9, passes=2, batch=1500, seed=7, rule=0)
+    g_ref, e_ref = oracle.vamana_build(oracle.lvq_encode(Y, mu, 8), **kw)
+    idx = lv.Index(0).set_primary(t(Y), t(mu), 8, d)
+    idx.build_graph(**kw)
+    idx.sync_status()
+    g, e = idx.get_graph()
+    assert e == e_ref
+    np.testing.assert_array_equal(g.cpu().numpy(), g_ref)
