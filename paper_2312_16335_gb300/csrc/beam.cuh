@@ -1074,7 +1074,8 @@ int launch_search_block4(const BeamParams &p, int nc, size_t smem, cudaStream_t 
 int launch_build_search(const BeamParams &p, int bits, int nc, int block, size_t smem, int num_sms,
                         cudaStream_t st);
 // scores the candidates the RERANK beam kernel handed over (p.cand, p.cand_n) and writes p.ids / p.scores
-int launch_rerank(const BeamParams &p, cudaStream_t st);
+constexpr int RR_TRIES = 1000;  // a wait for record copies gives up after as many tries (a second)
+int launch_rerank(const BeamParams &p, cudaStream_t st, int tries = RR_TRIES);
 
 // The search's launch shape (api.cu): beam / visited-cache / candidate capacities, width, warps and
 // queries per warp (p.Lcap .. p.qpw) from the index and the caller's parameters, the block size and
