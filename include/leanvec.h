@@ -453,7 +453,8 @@ typedef struct {
  * unreduced query and the best k written, sorted by score (ties -> smaller id), to
  * ids/scores (m x ldo, device); the rest of each row (fewer than k reachable
  * candidates, or k < ldo) is filled with -1 / -inf.  Reported scores are the
- * decoded inner products (secondary after rerank, primary otherwise).
+ * decoded inner products (secondary after rerank, primary otherwise).  A score that is not a
+ * number (NaN in the query, infinities or NaN behind a record) counts and is reported as -inf.
  * Streams: the work is ordered after `stream`'s earlier work and `stream`'s later
  * work waits for all of it.  With rerank and m above one wave of the beam kernel's
  * resident query slots (and not a multiple of it), the queries past 90 % of the last

@@ -679,7 +679,7 @@ __global__ void __launch_bounds__(256, 3) beam_kernel(const BeamParams p) {
             ps.score(cI, cS, 1, lane);
             __syncwarp();
             if (lane == 0) {
-                bS[0] = fmaxf(cS[0], -INFINITY);  // NaN (a query with NaN) ranks last: keys stay ordered
+                bS[0] = fmaxf(cS[0], -INFINITY);  // NaN ranks last: keys stay ordered
                 bI[0] = entry;
                 ctl[1] = 1;
                 ctl[2] = 0;

@@ -66,7 +66,7 @@ __global__ void __launch_bounds__(BB_T) beam_block_kernel(const BeamParams p) {
         ps.score(wI, wS, 1, lane);
         __syncwarp();
         if (lane == 0) {
-            bS[0] = fmaxf(wS[0], -INFINITY);  // NaN (a query with NaN) ranks last: keys stay ordered
+            bS[0] = fmaxf(wS[0], -INFINITY);  // NaN ranks last: keys stay ordered
             bI[0] = entry;
             s_cnt[0] = 0;
         }

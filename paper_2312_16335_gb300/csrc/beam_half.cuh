@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(320, 2) beam_half_kernel(const BeamParams p) {
             __syncwarp();
             if (fresh) {
                 if (hl == 0) {
-                    bS[0] = cS[0];
+                    bS[0] = fmaxf(cS[0], -INFINITY);  // NaN ranks last: keys stay ordered (see beam_kernel)
                     bI[0] = entry;
                 }
                 size = 1;
@@ -403,7 +403,7 @@ __global__ void __launch_bounds__(320, 2) beam_half_kernel(const BeamParams p) {
                 id[e] = 0;
                 pos[e] = 0;
                 if (jj[e] < cnt) {
-                    sc[e] = cS[jj[e]];
+                    sc[e] = fmaxf(cS[jj[e]], -INFINITY);
                     id[e] = cI[jj[e]];
                     valid[e] = !full || key_better(sc[e], id[e], tS, tI);
                 }

@@ -345,7 +345,7 @@ __global__ void __launch_bounds__(32 * RR_WARPS) rerank_kernel(const RerankParam
         for (int o = 4; o; o >>= 1) x += __shfl_xor_sync(FULL, x, o);
         const int u = lane >> 3;
         if ((lane & 7) == 0 && b + u < nr) {
-            const float f = sc.finish(x, rec + u * p.rec_bytes);
+            const float f = fmaxf(sc.finish(x, rec + u * p.rec_bytes), -INFINITY);  // NaN ranks last, as in the beam
             rS[b + u] = f;
             rK[b + u] = (unsigned long long)order_key(f) << 32 | (unsigned)~rI[b + u];
         }
