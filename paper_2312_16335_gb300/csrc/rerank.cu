@@ -31,7 +31,7 @@ struct RerankParams {
     int rec_bytes;   // bytes of a record that are read (codes and constants)
     const float *Q;  // unreduced queries m x D
     int D;
-    const float *smean;    // secondary mean mu (D) or NULL: cQ = <q, mu>, sQ = sum q per query
+    const float *smean;    // secondary mean mu (D): cQ = <q, mu>, sQ = sum q per query; NULL with FP16 records
     const int4 *desc;      // per query (k, L, r, max_hops) or NULL
     int4 uni;
     int64_t m;
@@ -396,6 +396,7 @@ static int launch_rerank_m(const BeamParams &bp, const RerankParams &p, cudaStre
             default: return fail(LV_ERR_ARG, "rerank: FP16 secondaries longer than 1024 dimensions");
         }
     }
+    if (!p.smean) return fail(LV_ERR_STATE, "rerank: LVQ-8 secondaries without their mean");
     return go_rerank<SecIntScorer<L2>>(p, st);
 }
 
