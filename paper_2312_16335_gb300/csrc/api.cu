@@ -224,8 +224,7 @@ int launch_beam_search(const lv_index *idx, const BeamParams &p, int block, size
 
 // A store's buffer of `want` bytes: the one the index holds when it is exactly that large, else a new
 // one.  A re-encode of the same shape would otherwise spend more time in cudaFree and cudaMalloc than
-// in its kernels (10k x 128: about 0.5 of 0.6 ms).  Every entry point that comes here first
-// synchronises the device, as cudaFree did, so no search of the old store is under way.
+// in its kernels (10k x 128: about 0.5 of 0.6 ms).  Every entry point that comes here calls quiesce first.
 template <class T>
 static cudaError_t store_buffer(T **p, size_t *have, size_t want) {
     if (*p && *have == want) return cudaSuccess;
@@ -236,6 +235,10 @@ static cudaError_t store_buffer(T **p, size_t *have, size_t want) {
     if (e == cudaSuccess) *have = want;
     return e;
 }
+
+// Before a held buffer is written again: waits until no search of it can be under way on any stream, as
+// cudaFree does before it frees.  An index that holds none has nothing to wait for.
+static cudaError_t quiesce(const void *held) { return held ? cudaDeviceSynchronize() : cudaSuccess; }
 
 extern "C" {
 
@@ -483,7 +486,7 @@ int leanvec_set_primary(lv_index *idx, const float *Y, int64_t n, int d, const f
     if (bits != 4 && bits != 8) return fail(LV_ERR_ARG, "set_primary: bits must be 4 or 8");
     DeviceGuard g(idx->device);
     if (!g.ok) return fail(LV_ERR_CUDA, "set_primary: cannot select device");
-    LV_CUDA(cudaDeviceSynchronize());
+    LV_CUDA(quiesce(idx->prim));
     if (idx->n != n) drop_secondary(idx);
     return set_primary_impl(idx, Y, n, d, mean, bits, D, (cudaStream_t)stream);
 }
@@ -494,7 +497,7 @@ int leanvec_set_secondary(lv_index *idx, const float *X, int64_t n, int D, const
     if (n != idx->n || D != idx->D) return fail(LV_ERR_ARG, "set_secondary: n and D must match the primary store");
     DeviceGuard g(idx->device);
     if (!g.ok) return fail(LV_ERR_CUDA, "set_secondary: cannot select device");
-    LV_CUDA(cudaDeviceSynchronize());
+    LV_CUDA(quiesce(idx->sec));
     return set_secondary_impl(idx, X, n, D, mean, 8, (cudaStream_t)stream);
 }
 
@@ -517,7 +520,7 @@ int leanvec_encode(lv_index *idx, const float *X, int64_t n, int D, const float 
     // buffers of another size go first: the new stores never sit beside the old ones
     rec_geom(d, primary_bits, pg, idx->metric);
     if (secondary_bits) rec_geom(D, secondary_bits, sg, idx->metric);
-    LV_TRYC(cudaDeviceSynchronize());
+    LV_TRYC(quiesce(idx->prim));
     if (idx->prim_b != (size_t)n * pg.stride || idx->pmean_b != sizeof(float) * d) drop_primary(idx);
     if (!secondary_bits || idx->sec_b != (size_t)n * sg.stride) drop_secondary(idx);
     forget_primary(idx);
