@@ -463,36 +463,36 @@ def autotune(index: "Index", Q: torch.Tensor, A: torch.Tensor | None, k: int, L:
              warps=(4, 8), hash_slots=(512, 1024, 2048, 4096), queries_per_warp=(1, 2), reps: int = 3) -> dict:
     """Pick the launch shape (queries per warp, warps per block, i.e. queries per CTA) and the
     visited-cache size for this batch by timing each candidate with CUDA events (two queries per
-    warp with the block sizes of HALF_WARPS, where the index and width allow it).  None of the
-    knobs changes the result (the visited cache is exact-preserving), only occupancy versus
-    re-scoring."""
+    warp with the block sizes of HALF_WARPS, where the index and width allow it).  The first candidate
+    leaves all of them to the library (zeros; with 1 in queries_per_warp), whose shapes for small
+    batches and long walks no explicit values name.  None of the knobs changes the result (the
+    visited cache is exact-preserving), only occupancy versus re-scoring."""
     best = None
     table = []
+    shapes = [(0, 0, 0)] * (1 in queries_per_warp)
+    shapes += [(qpw, w, h) for qpw in queries_per_warp for w in (HALF_WARPS if qpw == 2 else warps) for h in hash_slots
+               if h >= 2 * ((L + 31) // 32 * 32)]
     ldo = k
     ids = torch.empty((Q.shape[0], ldo), dtype=torch.int32, device=index.device)
     sc = torch.empty((Q.shape[0], ldo), dtype=torch.float32, device=index.device)
-    for qpw in queries_per_warp:
-        for w in (HALF_WARPS if qpw == 2 else warps):
-            for h in hash_slots:
-                if h < 2 * ((L + 31) // 32 * 32):
-                    continue
-                try:
-                    run = lambda: index.search(Q, A, k=k, L=L, rerank=rerank, desc=desc, ldo=ldo, out=(ids, sc),
-                                               width=width, projection=projection, hash_slots=h, warps_per_block=w,
-                                               queries_per_warp=qpw)
-                    run()
-                    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-                    e0.record()
-                    for _ in range(reps):
-                        run()
-                    e1.record()
-                    torch.cuda.synchronize()
-                    ms = e0.elapsed_time(e1) / reps
-                except LeanVecError:
-                    continue
-                table.append({"queries_per_warp": qpw, "warps_per_block": w, "hash_slots": h, "ms": ms})
-                if best is None or ms < best["ms"]:
-                    best = table[-1]
+    for qpw, w, h in shapes:
+        try:
+            run = lambda: index.search(Q, A, k=k, L=L, rerank=rerank, desc=desc, ldo=ldo, out=(ids, sc),
+                                       width=width, projection=projection, hash_slots=h, warps_per_block=w,
+                                       queries_per_warp=qpw)
+            run()
+            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            e0.record()
+            for _ in range(reps):
+                run()
+            e1.record()
+            torch.cuda.synchronize()
+            ms = e0.elapsed_time(e1) / reps
+        except LeanVecError:
+            continue
+        table.append({"queries_per_warp": qpw, "warps_per_block": w, "hash_slots": h, "ms": ms})
+        if best is None or ms < best["ms"]:
+            best = table[-1]
     return {"best": best, "table": table}
 
 
@@ -513,7 +513,9 @@ def autotune_uneven(index: "Index", Q: torch.Tensor, A: torch.Tensor | None, des
     For every launch of every plan the fastest warps per query (`teams`, dividing `width`), queries
     per warp (two with one warp per query, where the index allows it, with the block sizes of
     HALF_WARPS), visited-cache slots (0 = the library's default) and warps per block are picked by
-    timing the launch alone with CUDA events; the plan with the smallest total wins.  None of the knobs or
+    timing the launch alone with CUDA events, beside the library's own choice of all of them (listed
+    with queries_per_warp 0; when 1 is in `teams` and `queries_per_warp`); the plan with the smallest
+    total wins.  None of the knobs or
     plans changes a query's result.  Returns {"plan": name, "order": the permutation (device,
     int64) of the winning plan, "classes": its launches [{slice, L range, queries, k / L / rerank
     maxima, capacity, the chosen knobs, ms, qps}], "plans": {name: total ms}, "table": every timed
@@ -530,35 +532,32 @@ def autotune_uneven(index: "Index", Q: torch.Tensor, A: torch.Tensor | None, des
         dc = ds[sl]
         kmax, Lmax, rmax = (int(dc[:, j].max()) for j in range(3))
         best = None
-        shapes = [(T, 1) for T in teams] + [(1, 2)] * (2 in queries_per_warp)
-        for T, qpw in shapes:
+        shapes = [(1, 0, 0, 0)] * (1 in teams and 1 in queries_per_warp)
+        for T, qpw in [(T, 1) for T in teams] + [(1, 2)] * (2 in queries_per_warp):
             if width % T or (qpw == 1 and 1 not in queries_per_warp):
                 continue
-            for h in hash_slots:
-                if h and h < 2 * ((Lmax + 31) // 32 * 32):
-                    continue
-                for w in (HALF_WARPS if qpw == 2 else warps):
-                    if w % T:
-                        continue
-                    kw = dict(k=kmax, L=Lmax, rerank=rmax, desc=dc, ldo=ldo, out=(ids[sl], sc[sl]), width=width,
-                              projection=projection, hash_slots=h, warps_per_block=w, warps_per_query=T,
-                              queries_per_warp=qpw)
-                    try:
-                        index.search(Qs[sl], A, **kw)
-                        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-                        e0.record()
-                        for _ in range(reps):
-                            index.search(Qs[sl], A, **kw)
-                        e1.record()
-                        torch.cuda.synchronize(dev)
-                        ms = e0.elapsed_time(e1) / reps
-                    except LeanVecError:
-                        continue
-                    row = {"plan": name, "launch": c, "warps_per_query": T, "queries_per_warp": qpw,
-                           "hash_slots": h, "warps_per_block": w, "ms": ms}
-                    table.append(row)
-                    if best is None or ms < best["ms"]:
-                        best = row
+            shapes += [(T, qpw, h, w) for h in hash_slots if not h or h >= 2 * ((Lmax + 31) // 32 * 32)
+                       for w in (HALF_WARPS if qpw == 2 else warps) if w % T == 0]
+        for T, qpw, h, w in shapes:
+            kw = dict(k=kmax, L=Lmax, rerank=rmax, desc=dc, ldo=ldo, out=(ids[sl], sc[sl]), width=width,
+                      projection=projection, hash_slots=h, warps_per_block=w, warps_per_query=T if qpw else 0,
+                      queries_per_warp=qpw)
+            try:
+                index.search(Qs[sl], A, **kw)
+                e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                e0.record()
+                for _ in range(reps):
+                    index.search(Qs[sl], A, **kw)
+                e1.record()
+                torch.cuda.synchronize(dev)
+                ms = e0.elapsed_time(e1) / reps
+            except LeanVecError:
+                continue
+            row = {"plan": name, "launch": c, "warps_per_query": T, "queries_per_warp": qpw,
+                   "hash_slots": h, "warps_per_block": w, "ms": ms}
+            table.append(row)
+            if best is None or ms < best["ms"]:
+                best = row
         n_c = sl.stop - sl.start
         return {"slice": (sl.start, sl.stop), "L_range": (lo, hi), "queries": n_c, "k_max": kmax, "L_max": Lmax,
                 "rerank_max": rmax, "beam_capacity": (Lmax + 31) // 32 * 32,
@@ -615,11 +614,11 @@ class UnevenGraph:
         self.calls = []
         for c in plan["classes"]:
             sl = slice(*c["slice"])
+            qpw = c.get("queries_per_warp", 1)
             self.calls.append((sl, dict(k=c["k_max"], L=c["L_max"], rerank=c["rerank_max"], desc=self.ds[sl], ldo=ldo,
                                         out=(self.ids[sl], self.scores[sl]), width=width, projection=projection,
                                         hash_slots=c["hash_slots"], warps_per_block=c["warps_per_block"],
-                                        warps_per_query=c["warps_per_query"],
-                                        queries_per_warp=c.get("queries_per_warp", 1))))
+                                        warps_per_query=c["warps_per_query"] if qpw else 0, queries_per_warp=qpw)))
         s = torch.cuda.Stream(device=dev)
         s.wait_stream(torch.cuda.current_stream(dev))
         with torch.cuda.stream(s):
