@@ -438,7 +438,9 @@ typedef struct {
                                 with queries_per_warp 2 */
 } lv_search_params;
 
-/* Per-query counters (device, m entries) when stats != NULL. */
+/* Per-query counters (device, m entries) when stats != NULL.  Asking for them keeps a warp per query where
+ * a small batch would have a block per query (see warps_per_block): the answers and `hops` are the same, but
+ * `scored` is that launch's, whose visited cache holds fewer ids than the block's 4096. */
 typedef struct {
     int32_t hops;    /* beam expansions */
     int32_t scored;  /* primary records scored (re-scores of evicted visited ids included) */

@@ -103,7 +103,9 @@ int index_num_sms(lv_index *idx) { return idx->num_sms; }
 // Queries per SM up to which a batch runs with a block per query.  Time of a warp per query over that of a
 // block (200k x 768, L = 128 / 1M x 200, L = 300 / L2 200k x 960, L = 72 / 10k x 128, L = 50): 100 queries 1.15 /
 // 1.33 / 1.30 / 1.11, 608 1.20 / 1.37 / 1.27 / 1.09, 912 (six per SM) 1.07 / 1.20 / 1.23 / 1.06, 1216 0.82 /
-// 0.86 / 1.13 / 1.01, 1520 0.83 / 0.87 / 0.84 / 0.97.
+// 0.86 / 1.13 / 1.01, 1520 0.83 / 0.87 / 0.84 / 0.97.  LVQ-4 (300k x 768), width 1 / 2: 912 queries 1.13 / 1.21 at
+// L = 64, 1.07 / 1.28 at 256, 1.08 / 1.13 at 512.  L = 512, LVQ-8 (200k x 768): 608 queries 1.08 / 1.16, 912 1.01 /
+// 1.08, the smallest gain of the shapes looked at.
 constexpr int BLOCK_QUERIES = 6;
 
 static int next_pow2(int x) {
