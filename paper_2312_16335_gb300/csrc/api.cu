@@ -201,8 +201,8 @@ int search_shape(const lv_index *idx, const lv_search_params *params, BeamParams
     if (open && !p.stats && idx->pbits != 32 && p.W <= 2 && p.m <= (int64_t)BLOCK_QUERIES * idx->num_sms) {
         p.qpw = 0;
         p.vbits = 32;
-        p.Hcap = 4096;
-        p.hbits = 12;  // log2(4096)
+        p.Hcap = BB_SLOTS;
+        p.hbits = 12;  // log2(BB_SLOTS)
         p.Rcap = (int)round_up(p.W * idx->R, 32);
         p.warp_smem = block_query_smem(p.Lcap, p.Hcap, p.Rcap, qbytes);
         *smem = (size_t)p.warp_smem;

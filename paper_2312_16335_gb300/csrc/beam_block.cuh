@@ -22,10 +22,14 @@
 namespace lv {
 
 constexpr int BB_WARPS = 4, BB_T = 32 * BB_WARPS;
+constexpr int BB_SLOTS = 4096;  // visited cache of a query
 
 // shared bytes of a block: beam (8 Lcap), visited cache (4 Hcap), ids and scores of the new records and
 // id, score and place of the candidates (20 Rcap), the scorer's query
-inline int block_query_smem(int Lcap, int Hcap, int Rcap, int qbytes) { return 8 * Lcap + 4 * Hcap + 20 * Rcap + qbytes; }
+constexpr int block_query_smem(int Lcap, int Hcap, int Rcap, int qbytes) {
+    return 8 * Lcap + 4 * Hcap + 20 * Rcap + qbytes;
+}
+static_assert(block_query_smem(LCAP_MAX, BB_SLOTS, CMAX, 2048) <= 47 * 1024, "fits without asking for more");
 
 template <class PS, int WT>
 __global__ void __launch_bounds__(BB_T) beam_block_kernel(const BeamParams p) {
@@ -316,7 +320,6 @@ __global__ void __launch_bounds__(BB_T) beam_block_kernel(const BeamParams p) {
 template <class PS, int WT>
 int launch_block(const BeamParams &p, size_t smem, cudaStream_t st) {
     auto k = beam_block_kernel<PS, WT>;
-    LV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     if (p.slots) {  // every query has its block at once: no waves to cut the batch by
         *p.slots = INT64_MAX;
         return LV_OK;

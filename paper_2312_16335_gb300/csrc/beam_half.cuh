@@ -615,7 +615,7 @@ __global__ void __launch_bounds__(320, 2) beam_half_kernel(const BeamParams p) {
 template <int NC, int BITS, bool L2, int WT>
 static int half_go(const BeamParams &p, int block, size_t smem, int num_sms, cudaStream_t st) {
     auto k = beam_half_kernel<NC, BITS, L2, WT>;
-    LV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LV_CUDA(allow_smem(k, 0));
     LV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     int per_sm = 0;
     LV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem));

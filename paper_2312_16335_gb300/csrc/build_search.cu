@@ -7,7 +7,7 @@ namespace lv {
 template <int NC, int BITS, bool L2>
 static int go(const BeamParams &p, int block, size_t smem, int num_sms, cudaStream_t st) {
     auto k = beam_kernel<BuildScorer<NC, BITS, L2>, true, false, 1>;
-    LV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LV_CUDA(allow_smem(k, 0));
     LV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     int per_sm = 0;
     LV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem));
@@ -23,7 +23,7 @@ static int go(const BeamParams &p, int block, size_t smem, int num_sms, cudaStre
 template <int BITS, bool L2>
 static int go_warp(const BeamParams &p, int block, size_t smem, int num_sms, cudaStream_t st) {
     auto k = beam_kernel<BuildWarpScorer<BITS, L2>, true, false, 1>;
-    LV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LV_CUDA(allow_smem(k, 0));
     LV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     int per_sm = 0;
     LV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem));

@@ -41,6 +41,20 @@ void tmp_free(void *p, cudaStream_t st);
         if (_e != cudaSuccess) return ::lv::cuda_fail(_e, what);   \
     } while (0)
 
+// Lets `kernel` take the dynamic shared memory that a block has beside the kernel's static arrays
+// (static_bytes; -1: ask).  The limit belongs to the kernel and not to a launch: with one call's own size
+// there, another thread's larger launch of the kernel, under way at the time, would fail.
+template <class K>
+inline cudaError_t allow_smem(K *kernel, int static_bytes = -1) {
+    if (static_bytes < 0) {
+        cudaFuncAttributes a;
+        const cudaError_t e = cudaFuncGetAttributes(&a, (const void *)kernel);
+        if (e != cudaSuccess) return e;
+        static_bytes = (int)a.sharedSizeBytes;
+    }
+    return cudaFuncSetAttribute((const void *)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024 - static_bytes);
+}
+
 inline int64_t round_up(int64_t x, int64_t a) { return (x + a - 1) / a * a; }
 
 // Record geometry of an LVQ / float32 record (see leanvec.h).  LVQ records of an L2 index carry a

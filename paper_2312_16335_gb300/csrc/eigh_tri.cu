@@ -778,7 +778,7 @@ int eigh_top(const double *K, int D, int nout, double *evals, double *evecs, cud
                                             : (const void *)tridiag_sm_kernel<16>;
         const size_t sm = in_sm ? ssm : tsm;
         const int threads = in_sm ? TS_T : TRI_THREADS, blocks = in_sm ? gs : sms;
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess ||
+        if (allow_smem(kern) != cudaSuccess ||
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, sm) != cudaSuccess || per_sm < 1) {
             rc = fail(LV_ERR_CUDA, "eigh_top: cannot size the tridiagonalisation");
             goto done;
@@ -819,8 +819,8 @@ int eigh_top(const double *K, int D, int nout, double *evals, double *evecs, cud
         lo -= pad;
         hi += pad;
         const double pivmin = DBL_MIN * std::max(1.0, e2max);
-        if (cudaFuncSetAttribute(bisect_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bsm) != cudaSuccess ||
-            cudaFuncSetAttribute(inviter_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ism) != cudaSuccess) {
+        if (allow_smem(bisect_kernel) != cudaSuccess ||
+            allow_smem(inviter_kernel) != cudaSuccess) {
             rc = fail(LV_ERR_CUDA, "eigh_top: shared-memory attribute failed");
             goto done;
         }

@@ -561,7 +561,7 @@ static int jacobi_cluster(double *A, double *V, int Dp, int *sweeps_dev, double2
     const int rows = (Dp + JC_CL - 1) / JC_CL;
     const size_t smem = sizeof(double) * 2 * (size_t)rows * Dp;
     auto go = [&](auto kern, int threads) -> int {
-        LV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        LV_CUDA(allow_smem(kern));
         LV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(JC_CL);
@@ -653,7 +653,7 @@ int eigh_impl(const double *K, int D, int nout, double *evals, double *evecs, cu
     // one sweep = Dp - 1 rounds of (rotation angles, fused round); captured once into a CUDA
     // graph (launched per sweep), else launched directly
     if (fused && Dp * 32 > 48 * 1024 &&
-        cudaFuncSetAttribute(jacobi_round_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Dp * 32) != cudaSuccess) {
+        allow_smem(jacobi_round_kernel) != cudaSuccess) {
         cudaGetLastError();
         fused = false;
     }

@@ -1609,10 +1609,10 @@ static int gemm_tc(int fp8, const void *A, int64_t M, int64_t lda, const void *B
     const size_t sm = tc_smem(BN);
     dim3 grid((unsigned)((M + TC_BM - 1) / TC_BM), (unsigned)((N + BN - 1) / BN), (unsigned)splits);
     if (fp8) {
-        LV_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        LV_CUDA(allow_smem(gemm_tc_kernel<1>));
         gemm_tc_kernel<1><<<grid, 128, sm, st>>>(ta, tb, p);
     } else {
-        LV_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        LV_CUDA(allow_smem(gemm_tc_kernel<0>));
         gemm_tc_kernel<0><<<grid, 128, sm, st>>>(ta, tb, p);
     }
     LV_CHECK_LAUNCH("gemm_tc_kernel");
@@ -1768,7 +1768,7 @@ static int pair_tf32_launch(const float *Ah, const float *Al, int64_t M, int64_t
     const int kps = split_kps(K, splits, &used);
     // stages, barriers and flags, eight epilogue slabs (or the FP64 reduction slots), alignment slack
     const size_t sm = (size_t)PL_STAGES * 2 * (TC_BM + PL_BN) * 128 + 256 + 8 * 32 * 33 * 4 + 1024;
-    LV_CUDA(cudaFuncSetAttribute(pair_tf32_kernel<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    LV_CUDA(allow_smem(pair_tf32_kernel<MODE>));
     pair_tf32_kernel<MODE><<<grid, 64 + 32 * pair_epi_warps<MODE>(), sm, st>>>(tah, tal, tbh, tbl, (int)M, (int)N, (int)K, used, kps, o,
                                                          status);
     LV_CHECK_LAUNCH("pair_tf32_kernel");
@@ -1907,7 +1907,7 @@ int pair_flash(const __nv_bfloat16 *Rh, const __nv_bfloat16 *Rl, int64_t M, cons
     const int64_t items = ((M + TC_BM - 1) / TC_BM) * splits;
     const int grid = (int)std::min<int64_t>(items, std::max(1, sm_count()));
     const size_t sm = (size_t)PFL_STAGES * PFL_STAGE_BYTES + 256 + 1024;
-    LV_CUDA(cudaFuncSetAttribute(pair_flash_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    LV_CUDA(allow_smem(pair_flash_kernel));
     pair_flash_kernel<<<grid, 64 + 32 * PFL_EPI_WARPS, sm, st>>>(trh, trl, tch, tcl, tth, ttl, p);
     LV_CHECK_LAUNCH("pair_flash_kernel");
     return LV_OK;
@@ -2010,7 +2010,7 @@ static int project_bf16_fused(const float *X, int64_t n, int D, const float *P, 
     LV_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int64_t tiles = (n + TC_BM - 1) / TC_BM;
     const unsigned grid = (unsigned)std::min<int64_t>(tiles, sms);
-    LV_CUDA(cudaFuncSetAttribute(proj_f32in_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    LV_CUDA(allow_smem(proj_f32in_kernel));
     proj_f32in_kernel<<<grid, PF_THREADS, sm, st>>>(tx, tb, pp);
     LV_CHECK_LAUNCH("proj_f32in_kernel");
     return LV_OK;
@@ -2065,7 +2065,7 @@ int project_tf32x3(const float *X, int64_t n, int D, const float *P, int d, floa
     LV_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int64_t tiles = (n + TC_BM - 1) / TC_BM;
     const unsigned grid = (unsigned)std::min<int64_t>(tiles, sms);
-    LV_CUDA(cudaFuncSetAttribute(proj_tf32x3_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    LV_CUDA(allow_smem(proj_tf32x3_kernel));
     proj_tf32x3_kernel<<<grid, PF_THREADS, sm, st>>>(tx, tbh, tbl, pp);
     LV_CHECK_LAUNCH("proj_tf32x3_kernel");
     return LV_OK;
@@ -2433,7 +2433,7 @@ static int second_moment_f32in(const float *X, int64_t n, int D, float *K, int *
     p.status = status;
     const size_t sm = (size_t)GR_OSTAGES * GR_STAGE_BYTES + (size_t)GR_SLOTS * GR_SLOT_BYTES + 256 + 1024;
     int rc = LV_OK;
-    if (cudaFuncSetAttribute(gram_f32in_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm) != cudaSuccess)
+    if (allow_smem(gram_f32in_kernel) != cudaSuccess)
         rc = fail(LV_ERR_CUDA, "second_moment: shared-memory attribute failed");
     if (rc == LV_OK) {
         gram_f32in_kernel<<<(unsigned)(ranges * tiles), GR_THREADS, sm, st>>>(tx, p);

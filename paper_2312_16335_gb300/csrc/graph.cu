@@ -614,7 +614,7 @@ static int go_prune(const PruneParams &pp, unsigned grid, cudaStream_t st) {
     const int sm = prune_smem(pp.PMAX, pp.slot);
     if (grid == 0) return LV_OK;
     auto k = prune_kernel<BITS, MODE, L2, LONG, NT>;
-    LV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, sm));
+    LV_CUDA(allow_smem(k));
     k<<<grid, NT, sm, st>>>(pp);
     LV_CHECK_LAUNCH("prune_kernel");
     return LV_OK;

@@ -481,7 +481,7 @@ int launch_lvq_encode(const float *V, int64_t n, int dim, const float *mean, int
         const size_t smem = (size_t)dim * 8;
         const unsigned grid = (unsigned)std::min<int64_t>(blocks, (int64_t)sms * 8);
         auto go = [&](auto kern) -> int {
-            if (smem > 48 * 1024) LV_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            if (smem > 48 * 1024) LV_CUDA(allow_smem(kern));
             kern<<<grid, wpb * 32, smem, st>>>(V, n, dim, mean, rec, g.stride, g.code_bytes);
             LV_CHECK_LAUNCH("lvq_encode_vec_kernel");
             return LV_OK;

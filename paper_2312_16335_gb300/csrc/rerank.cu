@@ -375,11 +375,16 @@ __global__ void __launch_bounds__(32 * RR_WARPS) rerank_kernel(const RerankParam
     }
 }
 
+// the largest case: FP16 records of 1024 dimensions and L = LCAP_MAX
+constexpr int RR_SMEM_MAX = RR_WARPS * RR_STAGES * RR_GROUP * 2048 + 32 * 128 + 16 * LCAP_MAX;
+
 template <class SS>
 static int go_rerank(const RerankParams &p, cudaStream_t st) {
     const size_t smem = (size_t)RR_WARPS * RR_STAGES * RR_GROUP * p.rec_bytes + SS::query_bytes(p.sec_chunks) +
                         16 * (size_t)p.ldc;
-    LV_CUDA(cudaFuncSetAttribute(rerank_kernel<SS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // one limit for all sizes (see allow_smem), and none to set where every kernel may have as much
+    if (smem > 48 * 1024)
+        LV_CUDA(cudaFuncSetAttribute(rerank_kernel<SS>, cudaFuncAttributeMaxDynamicSharedMemorySize, RR_SMEM_MAX));
     rerank_kernel<SS><<<(unsigned)p.m, 32 * RR_WARPS, smem, st>>>(p);
     LV_CHECK_LAUNCH("rerank_kernel");
     return LV_OK;

@@ -23,7 +23,7 @@ struct WarpAt {
 template <class K>
 int launch_persistent(K k, const BeamParams &p, int block, size_t smem, int num_sms, cudaStream_t st,
                       const char *name) {
-    LV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LV_CUDA(allow_smem(k, 0));
     LV_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100));
     int per_sm = 0;
     LV_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, block, smem));
