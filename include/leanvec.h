@@ -142,7 +142,8 @@ int leanvec_project(const float *X, int64_t n, int D, const float *P, int d, flo
 int leanvec_second_moment(const float *X, int64_t n, int D, float *K, int precision, lv_stream_t stream);
 
 /* Eigen-decomposition of a symmetric D x D FP64 matrix K (device) by cyclic
- * Jacobi rotations in FP64: evals (D, device, may be NULL) in descending order,
+ * Jacobi rotations in FP64 (up to 256 rows the angles, which steer the sweeps, come from float32;
+ * each rotation is orthogonal to FP64): evals (D, device, may be NULL) in descending order,
  * evecs (D x D, device) with row r the eigenvector of evals[r], its
  * largest-magnitude entry positive (first index on ties).  Synchronises `stream`. */
 int leanvec_eigh(const double *K, int D, double *evals, double *evecs, lv_stream_t stream);
@@ -152,7 +153,8 @@ int leanvec_eigh(const double *K, int D, double *evals, double *evecs, lv_stream
  * use: Householder reduction to tridiagonal form (all SMs, one cooperative launch), bisection on
  * Sturm counts for the nout largest eigenvalues, inverse iteration for their tridiagonal
  * eigenvectors (Gram-Schmidt among eigenvalues closer than 1e-5 of the largest magnitude), and
- * the back-transformation; FP64 throughout.  evals (nout, device, nullable) descending, evecs
+ * the back-transformation; FP64, after float32 has narrowed the eigenvalues' first intervals, whose
+ * ends FP64 checks.  evals (nout, device, nullable) descending, evecs
  * (nout x D, device) rows = unit eigenvectors with the largest-magnitude entry positive (first
  * index on ties), as leanvec_eigh.  Returns LV_ERR_TIMEOUT if a grid barrier of the reduction
  * gave up (seconds).  Synchronises `stream`.  leanvec_fit_id and leanvec_fit_ood use this path

@@ -9,7 +9,8 @@
 //      cluster);
 //   4. maps them back through the reflections (x = Q z, one block per eigenvector) and fixes the
 //      sign (largest-magnitude entry positive, first index on ties).
-// FP64 throughout.  Every grid-wide wait is bounded: a block that waits too long records
+// FP64, with float32 only where FP64 decides the result: three rounds of the multisection narrow an interval
+// whose ends an FP64 round then checks.  Reciprocals and roots as in fp64.cuh.  Every grid-wide wait is bounded: a block that waits too long records
 // ST_TIMEOUT and returns.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
@@ -21,6 +22,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "fp64.cuh"
 
 namespace lv {
 
@@ -71,24 +73,6 @@ __device__ bool grid_barrier(unsigned *count, volatile unsigned *gen, unsigned &
         __threadfence();
     }
     return __syncthreads_and(ok) != 0;
-}
-
-// FP64 on this chip: a warp instruction takes the pipe for 64 cycles, a division 550 and a root 585,
-// and extra warps on a scheduler only queue.  So the kernels below keep one warp per scheduler,
-// share no work redundantly between warps of a scheduler, and take reciprocals and roots from the
-// hardware's approximations (about 2^-20 relative) by one cubic step (error e^3, below 2^-58):
-//   1/x: y (1 + e + e^2), e = 1 - x y;   1/sqrt(x): y (1 + r/2 + 3 r^2/8), r = 1 - x y^2.
-__device__ __forceinline__ double fast_rcp(double x) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x, y, 1.0);
-    return fma(y, fma(e, e, e), y);
-}
-__device__ __forceinline__ double fast_rsqrt(double x) {
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double r = fma(-x * y, y, 1.0);
-    return fma(y * r, fma(0.375, r, 0.5), y);
 }
 
 // The grid barrier again, polled without sleeping on the arrival counter itself.

@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "common.cuh"
+#include "fp64.cuh"
 
 namespace lv {
 
@@ -311,35 +312,6 @@ __device__ __forceinline__ void st_cluster(uint32_t addr, int rank, double v) {
 }
 __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
-// v 2^-e as float32 (truncated; 0 below its range), e an exponent field >= v's: integer instructions only
-__device__ __forceinline__ float scaled_float(double v, int e) {
-    const int hi = __double2hiint(v), x = ((hi >> 20) & 0x7ff) - e + 127;
-    const unsigned m = ((unsigned)hi & 0xfffffu) << 3 | (unsigned)__double2loint(v) >> 29;
-    return x > 0 ? __uint_as_float(((unsigned)hi & 0x80000000u) | (unsigned)x << 23 | m) : 0.f;
-}
-// a float32 as FP64 (0 below its normal range), integer instructions only
-__device__ __forceinline__ double float_bits_to_double(float f) {
-    const unsigned u = __float_as_uint(f), x = (u >> 23) & 0xffu;
-    if (x == 0u) return 0.0;
-    return __hiloint2double((int)((u & 0x80000000u) | (x + 896u) << 20 | (u & 0x7fffffu) >> 3), (int)(u << 29));
-}
-
-// tangent t and cosine c of the rotation that (nearly) zeroes a_pq: rows p <- c (p - t q), q <- c (q + t p)
-__device__ __forceinline__ void jacobi_angle(double app, double aqq, double apq, double &t, double &c) {
-    const double d = aqq - app;
-    const int ed = (__double2hiint(d) >> 20) & 0x7ff, ex = (__double2hiint(apq) >> 20) & 0x7ff;
-    const int e = max(ed, ex);
-    const float theta = 0.5f * scaled_float(d, e) / scaled_float(apq, e);
-    const float tf = copysignf(1.0f / (fabsf(theta) + sqrtf(fmaf(theta, theta, 1.0f))), theta);
-    // no rotation for 0 / 0, a_pq below 2^-996 (about 1e-300) or entries that are not finite
-    t = fabsf(tf) <= 1.0f && ex > 27 && e < 0x7ff ? float_bits_to_double(tf) : 0.0;
-    const double u = fma(t, t, 1.0);
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(u));  // about 2^-20
-    const double r = fma(-u, y * y, 1.0);                     // y (1 + r / 2 + 3 r^2 / 8) is good to r^3
-    c = fma(y * r, fma(0.375, r, 0.5), y);
 }
 
 // pair k of round r on Dp (even) indices, as rr_pair, with 0 <= r < Dp - 1
