@@ -210,9 +210,9 @@ __device__ __forceinline__ unsigned score_key(float s) {
 __device__ __forceinline__ float key_score(unsigned k) {
     return __uint_as_float(k ^ ((k >> 31) ? 0x80000000u : 0xffffffffu));
 }
-// (score, id) in one word: the larger the better, ties by the smaller id
+// (score, id) in one word: the larger the better, ties by the smaller id; NaN as -infinity, as in the beam
 __device__ __forceinline__ unsigned long long pool_key(float s, int id) {
-    return (unsigned long long)score_key(s) << 32 | (unsigned)~id;
+    return (unsigned long long)score_key(fmaxf(s, -INFINITY)) << 32 | (unsigned)~id;
 }
 
 // Writes the values of the block's kept threads, in thread order, to dst[base ..) while they fit below
