@@ -472,70 +472,49 @@ struct BuildWarpScorer {
 };
 
 // --------------------------------------------------------------------------------
-// Whole-warp scorer for long records: float32 vectors (KIND 0, the full-dimensional
-// baseline) or LVQ-8 secondary records (KIND 1, the rerank).  U records per pass.
+// Whole-warp scorer for float32 vectors (the full-dimensional baseline).  U records per pass.
 // --------------------------------------------------------------------------------
-// L2 (float32 records): 2 <q, x> - ||x||^2, the norm summed from the record itself
-template <int NCW, int KIND, bool L2 = false>
+// L2: 2 <q, x> - ||x||^2, the norm summed from the record itself
+template <int NCW, bool L2 = false>
 struct WarpScorer {
-    static constexpr int CPC = KIND == 0 ? 4 : 16;
-    static constexpr int U = KIND == 0 ? (NCW > 4 ? 2 : 4) : 4;
-    float q[NCW][CPC];
-    float c0, s0;
+    static constexpr int U = NCW > 4 ? 2 : 4;
+    static constexpr int QBYTES = 0;
+    static constexpr bool PREFETCH = false;
+    float q[NCW][4];
     int CH;
     const uint8_t *base;
     int64_t stride;
 
-    // qrow: qlen valid floats (the rest read as 0)
-    __device__ __forceinline__ void setup_row(const float *qrow, int qlen, int chunks, const uint8_t *b,
-                                              int64_t st, float cc, float ss, int lane) {
-        CH = chunks;
-        base = b;
-        stride = st;
-        c0 = cc;
-        s0 = ss;
+    // padded queries, no constants
+    __device__ __forceinline__ void setup(const BeamParams &p, int64_t qi, int lane, void *, bool) {
+        const float *qrow = p.qp + qi * p.ldq;
+        CH = p.prim_chunks;
+        base = p.prim;
+        stride = p.prim_stride;
 #pragma unroll
         for (int t = 0; t < NCW; ++t) {
             const int c = lane + 32 * t;
 #pragma unroll
-            for (int e = 0; e < CPC; ++e) {
-                const int j = c * CPC + e;
-                q[t][e] = (c < CH && j < qlen) ? qrow[j] : 0.0f;
+            for (int e = 0; e < 4; ++e) {
+                const int j = c * 4 + e;
+                q[t][e] = (c < CH && j < p.ldq) ? qrow[j] : 0.0f;
             }
         }
-    }
-
-    static constexpr int QBYTES = 0;
-    static constexpr bool PREFETCH = false;
-    __device__ __forceinline__ void setup(const BeamParams &p, int64_t qi, int lane, void *, bool) {
-        // full-dimensional float32 search: padded queries, no constants
-        setup_row(p.qp + qi * p.ldq, p.ldq, p.prim_chunks, p.prim, p.prim_stride, 0.f, 0.f, lane);
     }
 
     __device__ __forceinline__ float dot1(const uint4 (&v)[NCW]) const {
         float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f, nn = 0.f;
 #pragma unroll
         for (int t = 0; t < NCW; ++t) {
-            if (KIND == 0) {
-                a0 = fmaf(q[t][0], __uint_as_float(v[t].x), a0);
-                a1 = fmaf(q[t][1], __uint_as_float(v[t].y), a1);
-                a2 = fmaf(q[t][2], __uint_as_float(v[t].z), a2);
-                a3 = fmaf(q[t][3], __uint_as_float(v[t].w), a3);
-                if (L2) {
-                    nn = fmaf(__uint_as_float(v[t].x), __uint_as_float(v[t].x), nn);
-                    nn = fmaf(__uint_as_float(v[t].y), __uint_as_float(v[t].y), nn);
-                    nn = fmaf(__uint_as_float(v[t].z), __uint_as_float(v[t].z), nn);
-                    nn = fmaf(__uint_as_float(v[t].w), __uint_as_float(v[t].w), nn);
-                }
-            } else {
-                const uint32_t w[4] = {v[t].x, v[t].y, v[t].z, v[t].w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    a0 = fmaf(q[t][4 * i + 0], byte_to_float<0>(w[i]), a0);
-                    a1 = fmaf(q[t][4 * i + 1], byte_to_float<1>(w[i]), a1);
-                    a2 = fmaf(q[t][4 * i + 2], byte_to_float<2>(w[i]), a2);
-                    a3 = fmaf(q[t][4 * i + 3], byte_to_float<3>(w[i]), a3);
-                }
+            a0 = fmaf(q[t][0], __uint_as_float(v[t].x), a0);
+            a1 = fmaf(q[t][1], __uint_as_float(v[t].y), a1);
+            a2 = fmaf(q[t][2], __uint_as_float(v[t].z), a2);
+            a3 = fmaf(q[t][3], __uint_as_float(v[t].w), a3);
+            if (L2) {
+                nn = fmaf(__uint_as_float(v[t].x), __uint_as_float(v[t].x), nn);
+                nn = fmaf(__uint_as_float(v[t].y), __uint_as_float(v[t].y), nn);
+                nn = fmaf(__uint_as_float(v[t].z), __uint_as_float(v[t].z), nn);
+                nn = fmaf(__uint_as_float(v[t].w), __uint_as_float(v[t].w), nn);
             }
         }
         const float ip = (a0 + a1) + (a2 + a3);
@@ -543,8 +522,6 @@ struct WarpScorer {
     }
 
     __device__ __forceinline__ void score(const int *ids, float *out, int cnt, int lane) const {
-        const int tot = CH + (KIND == 1 ? 1 : 0);
-        const int holder = CH & 31, tslot = CH >> 5;
         for (int b = 0; b < cnt; b += U) {
             uint4 v[U][NCW];
 #pragma unroll
@@ -554,7 +531,7 @@ struct WarpScorer {
 #pragma unroll
                 for (int t = 0; t < NCW; ++t) {
                     const int c = lane + 32 * t;
-                    v[u][t] = (c < tot && id >= 0) ? ldg_stream(r + 16 * c) : make_uint4(0, 0, 0, 0);
+                    v[u][t] = (c < CH && id >= 0) ? ldg_stream(r + 16 * c) : make_uint4(0, 0, 0, 0);
                 }
             }
 #pragma unroll
@@ -562,18 +539,6 @@ struct WarpScorer {
                 float s = dot1(v[u]);
 #pragma unroll
                 for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(FULL, s, o);
-                float dl = 0.f, lo = 0.f;
-                if (KIND == 1) {
-#pragma unroll
-                    for (int t = 0; t < NCW; ++t)
-                        if (t == tslot) {
-                            dl = __uint_as_float(v[u][t].x);
-                            lo = __uint_as_float(v[u][t].y);
-                        }
-                    dl = __shfl_sync(FULL, dl, holder);
-                    lo = __shfl_sync(FULL, lo, holder);
-                    s = fmaf(dl, s, fmaf(lo, s0, c0));
-                }
                 if (lane == 0 && b + u < cnt) out[b + u] = s;
             }
         }

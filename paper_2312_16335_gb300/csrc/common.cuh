@@ -101,13 +101,6 @@ __device__ __forceinline__ uint4 ldg_stream(const void *p) {
     return v;
 }
 
-// float(b) for the byte of w selected by SEL, exact: builds 2^23 + b and subtracts 2^23.
-template <int SEL>
-__device__ __forceinline__ float byte_to_float(uint32_t w) {
-    uint32_t bits = __byte_perm(w, 0x4B000000u, 0x7540u | SEL);
-    return __int_as_float((int)bits) - 8388608.0f;
-}
-
 // The exact build score <y_a, y_b> of two primaries (see leanvec.h): integer sums P and the
 // per-record terms combined by one fixed sequence of float32 operations (no FMA).
 __device__ __forceinline__ float build_pair_score(float mu2, float fdim, float da, float la, float Ga, float Ha,

@@ -10,8 +10,8 @@
 //   4. maps them back through the reflections (x = Q z, one block per eigenvector) and fixes the
 //      sign (largest-magnitude entry positive, first index on ties).
 // FP64, with float32 only where FP64 decides the result: three rounds of the multisection narrow an interval
-// whose ends an FP64 round then checks.  Reciprocals and roots as in fp64.cuh.  Every grid-wide wait is bounded: a block that waits too long records
-// ST_TIMEOUT and returns.
+// whose ends an FP64 round then checks.  Reciprocals and roots as in fp64.cuh.  Every grid-wide wait is
+// bounded: a block that waits too long records ST_TIMEOUT and returns.
 #include <cooperative_groups.h>
 #include <cuda_runtime.h>
 

@@ -24,28 +24,27 @@ int launch_gram_fp32(const float *X, int64_t n, int D, float *K, cudaStream_t st
 int second_moment_bf16(const float *X, int64_t n, int D, float *K, int *status, cudaStream_t st);
 
 // ------------------------------------------------------------- small GEMM
-// C (M x N, ldc) = alpha * op(A) op(B) + beta * C, float32 or float64, op = transpose
+// C (M x N, ldc) = alpha * op(A) op(B) + beta * C in float32, op = transpose
 // when the flag is set (A is M x K, or K x M when transposed; B is K x N or N x K).
-template <typename T>
-__global__ void __launch_bounds__(256) gemm_small_kernel(int M, int N, int K, T alpha, const T *__restrict__ A, int lda,
-                                                         bool ta, const T *__restrict__ B, int ldb, bool tb, T beta,
-                                                         T *__restrict__ C, int ldc) {
-    __shared__ T As[16][65];
-    __shared__ T Bs[16][65];
+__global__ void __launch_bounds__(256) gemm_small_kernel(int M, int N, int K, float alpha, const float *__restrict__ A,
+                                                         int lda, bool ta, const float *__restrict__ B, int ldb, bool tb,
+                                                         float beta, float *__restrict__ C, int ldc) {
+    __shared__ float As[16][65];
+    __shared__ float Bs[16][65];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
     const int r0 = blockIdx.y * 64, c0 = blockIdx.x * 64;
-    T acc[4][4] = {};
+    float acc[4][4] = {};
     for (int k0 = 0; k0 < K; k0 += 16) {
         for (int t = threadIdx.x; t < 16 * 64; t += 256) {
             const int kk = t / 64, i = t % 64;
             const int r = r0 + i, k = k0 + kk, c = c0 + i;
-            As[kk][i] = (r < M && k < K) ? (ta ? A[(int64_t)k * lda + r] : A[(int64_t)r * lda + k]) : T(0);
-            Bs[kk][i] = (c < N && k < K) ? (tb ? B[(int64_t)c * ldb + k] : B[(int64_t)k * ldb + c]) : T(0);
+            As[kk][i] = (r < M && k < K) ? (ta ? A[(int64_t)k * lda + r] : A[(int64_t)r * lda + k]) : 0.f;
+            Bs[kk][i] = (c < N && k < K) ? (tb ? B[(int64_t)c * ldb + k] : B[(int64_t)k * ldb + c]) : 0.f;
         }
         __syncthreads();
 #pragma unroll
         for (int kk = 0; kk < 16; ++kk) {
-            T a[4], b[4];
+            float a[4], b[4];
 #pragma unroll
             for (int u = 0; u < 4; ++u) a[u] = As[kk][ty * 4 + u];
 #pragma unroll
@@ -65,17 +64,16 @@ __global__ void __launch_bounds__(256) gemm_small_kernel(int M, int N, int K, T 
         for (int v = 0; v < 4; ++v) {
             const int c = c0 + tx * 4 + v;
             if (c >= N) continue;
-            T *o = C + (int64_t)r * ldc + c;
-            *o = alpha * acc[u][v] + (beta == T(0) ? T(0) : beta * *o);
+            float *o = C + (int64_t)r * ldc + c;
+            *o = alpha * acc[u][v] + (beta == 0.f ? 0.f : beta * *o);
         }
     }
 }
 
-template <typename T>
-static int gemm_small(int M, int N, int K, T alpha, const T *A, int lda, bool ta, const T *B, int ldb, bool tb, T beta,
-                      T *C, int ldc, cudaStream_t st) {
+static int gemm_small(int M, int N, int K, float alpha, const float *A, int lda, bool ta, const float *B, int ldb,
+                      bool tb, float beta, float *C, int ldc, cudaStream_t st) {
     dim3 grd((N + 63) / 64, (M + 63) / 64);
-    gemm_small_kernel<T><<<grd, 256, 0, st>>>(M, N, K, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc);
+    gemm_small_kernel<<<grd, 256, 0, st>>>(M, N, K, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc);
     LV_CHECK_LAUNCH("gemm_small_kernel");
     return LV_OK;
 }
@@ -222,12 +220,12 @@ static int ood_loss_dev(OodCtx &c, const float *A, const float *B, double *f) {
     const int D = c.D, d = c.d;
     int rc;
     // t1 = A K_Q, s1 = t1 A^T ; t2 = B K_X, s2 = t2 B^T
-    if ((rc = gemm_small<float>(d, D, D, 1.f, A, D, false, c.KQ, D, false, 0.f, c.t1, D, c.st))) return rc;
-    if ((rc = gemm_small<float>(d, d, D, 1.f, c.t1, D, false, A, D, true, 0.f, c.s1, d, c.st))) return rc;
-    if ((rc = gemm_small<float>(d, D, D, 1.f, B, D, false, c.KX, D, false, 0.f, c.t2, D, c.st))) return rc;
-    if ((rc = gemm_small<float>(d, d, D, 1.f, c.t2, D, false, B, D, true, 0.f, c.s2, d, c.st))) return rc;
+    if ((rc = gemm_small(d, D, D, 1.f, A, D, false, c.KQ, D, false, 0.f, c.t1, D, c.st))) return rc;
+    if ((rc = gemm_small(d, d, D, 1.f, c.t1, D, false, A, D, true, 0.f, c.s1, d, c.st))) return rc;
+    if ((rc = gemm_small(d, D, D, 1.f, B, D, false, c.KX, D, false, 0.f, c.t2, D, c.st))) return rc;
+    if ((rc = gemm_small(d, d, D, 1.f, c.t2, D, false, B, D, true, 0.f, c.s2, d, c.st))) return rc;
     // t3 = t2 K_Q = B K_X K_Q ; tr(K_Q A^T B K_X) = <A, B K_X K_Q>_F
-    if ((rc = gemm_small<float>(d, D, D, 1.f, c.t2, D, false, c.KQ, D, false, 0.f, c.t3, D, c.st))) return rc;
+    if ((rc = gemm_small(d, D, D, 1.f, c.t2, D, false, c.KQ, D, false, 0.f, c.t3, D, c.st))) return rc;
     LV_CUDA(cudaMemsetAsync(c.acc, 0, 2 * sizeof(double), c.st));
     trace_prod_kernel<<<16, 256, 0, c.st>>>(c.s1, c.s2, d, c.acc);
     frob_dot_kernel<<<64, 256, 0, c.st>>>(A, c.t3, (int64_t)d * D, c.acc + 1);
@@ -245,14 +243,14 @@ static int ood_loss_dev(OodCtx &c, const float *A, const float *B, double *f) {
 static int ood_grad_dev(OodCtx &c, const float *Y, const float *KY, const float *Z, const float *KZ, float *g) {
     const int D = c.D, d = c.d;
     int rc;
-    if ((rc = gemm_small<float>(d, D, D, 1.f, Y, D, false, KY, D, false, 0.f, c.t1, D, c.st))) return rc;  // Y K_Y
-    if ((rc = gemm_small<float>(d, d, D, 1.f, c.t1, D, false, Y, D, true, 0.f, c.s1, d, c.st))) return rc;  // Y K_Y Y^T
+    if ((rc = gemm_small(d, D, D, 1.f, Y, D, false, KY, D, false, 0.f, c.t1, D, c.st))) return rc;  // Y K_Y
+    if ((rc = gemm_small(d, d, D, 1.f, c.t1, D, false, Y, D, true, 0.f, c.s1, d, c.st))) return rc;  // Y K_Y Y^T
     // t2 = s1 Z - t1
-    if ((rc = gemm_small<float>(d, D, d, 1.f, c.s1, d, false, Z, D, false, 0.f, c.t2, D, c.st))) return rc;
+    if ((rc = gemm_small(d, D, d, 1.f, c.s1, d, false, Z, D, false, 0.f, c.t2, D, c.st))) return rc;
     axpby_kernel<<<(unsigned)(((int64_t)d * D + 255) / 256), 256, 0, c.st>>>(1.f, c.t2, -1.f, c.t1, (int64_t)d * D,
                                                                            c.t2);
     LV_CHECK_LAUNCH("axpby_kernel");
-    return gemm_small<float>(d, D, D, 2.f, c.t2, D, false, KZ, D, false, 0.f, g, D, c.st);
+    return gemm_small(d, D, D, 2.f, c.t2, D, false, KZ, D, false, 0.f, g, D, c.st);
 }
 
 // S = argmax_{||S||_op <= 1} <S, C> = polar factor (C C^T)^{-1/2} C (FP64 eig of C C^T)
@@ -526,10 +524,10 @@ int leanvec_fit_ood(const float *X, int64_t n, const float *Q, int64_t m, int D,
                     axpby_kernel<<<(unsigned)((dD + 255) / 256), 256, 0, st>>>(1.f, c.S, -1.f, Z, (int64_t)dD, Dl);
                     double slope, curv;
                     if ((rc = red_frob(c, g, Dl, (int64_t)dD, &slope))) goto done;
-                    if ((rc = gemm_small<float>(d, D, D, 1.f, Y, D, false, KY, D, false, 0.f, c.t1, D, st))) goto done;
-                    if ((rc = gemm_small<float>(d, d, D, 1.f, c.t1, D, false, Y, D, true, 0.f, c.s1, d, st))) goto done;
-                    if ((rc = gemm_small<float>(d, D, D, 1.f, Dl, D, false, KZ, D, false, 0.f, c.t2, D, st))) goto done;
-                    if ((rc = gemm_small<float>(d, d, D, 1.f, c.t2, D, false, Dl, D, true, 0.f, c.s2, d, st))) goto done;
+                    if ((rc = gemm_small(d, D, D, 1.f, Y, D, false, KY, D, false, 0.f, c.t1, D, st))) goto done;
+                    if ((rc = gemm_small(d, d, D, 1.f, c.t1, D, false, Y, D, true, 0.f, c.s1, d, st))) goto done;
+                    if ((rc = gemm_small(d, D, D, 1.f, Dl, D, false, KZ, D, false, 0.f, c.t2, D, st))) goto done;
+                    if ((rc = gemm_small(d, d, D, 1.f, c.t2, D, false, Dl, D, true, 0.f, c.s2, d, st))) goto done;
                     if ((rc = red_frob(c, c.s1, c.s2, (int64_t)dd, &curv))) goto done;
                     step = curv > 0.0 ? std::min(1.0, std::max(0.0, -slope / (2.0 * curv))) : (slope < 0.0 ? 1.0 : 0.0);
                 }

@@ -17,7 +17,7 @@ struct LvqAt {
 template <int NCW>
 struct WarpAt {
     template <bool L2>
-    using S = WarpScorer<NCW, 0, L2>;
+    using S = WarpScorer<NCW, L2>;
 };
 
 template <class K>
