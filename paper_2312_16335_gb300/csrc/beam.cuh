@@ -156,7 +156,8 @@ struct LvqIntScorer {
     // the 128-byte lines holding a record's first and last byte are prefetched into L2 as soon as the
     // visited test admits its id, so that the scorer's passes after the first one find the record
     // there (all of it when it spans at most two lines, as the 192-byte records of d = 160 do)
-    static constexpr bool PREFETCH = true;
+    static constexpr bool PREFETCH = true, COPIES_APART = false;
+    static constexpr int BLOCKS = 3;  // 80 registers, 24 warps on an SM
     __device__ __forceinline__ int rec_bytes() const { return 16 * (CH + 1 + (L2 ? 1 : 0)); }
     const uint4 *lq;
     float cq, sq, scale;
@@ -336,7 +337,8 @@ struct BuildScorer {
     int64_t stride;
 
     static constexpr int QBYTES = 0;
-    static constexpr bool PREFETCH = true;
+    static constexpr bool PREFETCH = true, COPIES_APART = false;
+    static constexpr int BLOCKS = 3;  // 80 registers, 24 warps on an SM
     __device__ __forceinline__ int rec_bytes() const { return 16 * (CH + 1 + (L2 ? 1 : 0)); }
     __device__ __forceinline__ void setup(const BeamParams &p, int64_t qi, int lane, void *, bool) {
         CH = p.prim_chunks;
@@ -409,7 +411,8 @@ struct BuildScorer {
 template <int BITS, bool L2 = false>
 struct BuildWarpScorer {
     static constexpr int QBYTES = 0;
-    static constexpr bool PREFETCH = true;
+    static constexpr bool PREFETCH = true, COPIES_APART = false;
+    static constexpr int BLOCKS = 3;  // 80 registers, 24 warps on an SM
     __device__ __forceinline__ int rec_bytes() const { return 16 * (CH + 1 + (L2 ? 1 : 0)); }
     static constexpr int U = 4;
     uint4 qc[2];
@@ -479,7 +482,10 @@ template <int NCW, bool L2 = false>
 struct WarpScorer {
     static constexpr int U = NCW > 4 ? 2 : 4;
     static constexpr int QBYTES = 0;
-    static constexpr bool PREFETCH = false;
+    static constexpr bool PREFETCH = false, COPIES_APART = true;
+    // up to 128 dimensions fit 64 registers: 32 warps on an SM instead of 24 (20,000 queries on 100k x 128 with 72
+    // registers and 24 warps: 1.15 times as long)
+    static constexpr int BLOCKS = NCW == 1 ? 4 : 3;
     float q[NCW][4];
     int CH;
     const uint8_t *base;
@@ -567,6 +573,43 @@ __device__ __forceinline__ bool bucket_tag_free(const uint4 v, unsigned tag, int
     return true;
 }
 
+// Keeps the first copy of every id among the cv candidates of a round, in order; returns their number (one
+// warp).  Rare, and called out of line by the float32 scorers, whose queries and records leave no registers
+// for it: inlined it cost the walks of 768-dimensional records at width 2 13 to 16 % (12 bytes of spills and a
+// slower schedule for 0), while the LVQ scorers lose 1 % by the call.
+__device__ __forceinline__ int drop_copies(int *cI, float *cS, int *vPB, int cv, int lane) {
+    const unsigned lt = (1u << lane) - 1u;
+    int cv2 = 0;
+    for (int j0 = 0; j0 < cv; j0 += 32) {
+        const int j = j0 + lane;
+        bool keep = j < cv;
+        float s = 0.f;
+        int id = 0, pb = 0;
+        if (keep) {
+            s = cS[j];
+            id = cI[j];
+            pb = vPB[j] & 0xffff;
+            // copies before j: kept ones (already compacted) or of this chunk
+            for (int u = 0; u < cv2; ++u) keep &= cI[u] != id;
+            for (int u = j0; u < j; ++u) keep &= cI[u] != id;
+        }
+        const unsigned bal = __ballot_sync(FULL, keep);
+        __syncwarp();
+        if (keep) {
+            const int o = cv2 + __popc(bal & lt);
+            cI[o] = id;
+            cS[o] = s;
+            vPB[o] = pb;
+        }
+        cv2 += __popc(bal);
+        __syncwarp();
+    }
+    return cv2;
+}
+static __device__ __noinline__ int drop_copies_apart(int *cI, float *cS, int *vPB, int cv, int lane) {
+    return drop_copies(cI, cS, vPB, cv, lane);
+}
+
 // --------------------------------------------------------------------------------
 // The beam kernel.  A team of T = p.T warps serves one query: per round the W best
 // unexpanded beam members are the parents, warp w of the team expands parents
@@ -579,7 +622,7 @@ __device__ __forceinline__ bool bucket_tag_free(const uint4 v, unsigned tag, int
 // WT: the search width fixed at compile time (1 or 2; 0 = p.W, up to WMAX); TAGS: the visited
 // cache holds 16-bit tags in buckets of 8 (p.vbits = 16) instead of ids in buckets of 4
 template <class PS, bool BUILD, bool RERANK, int WT, bool TAGS = false>
-__global__ void __launch_bounds__(256, 3) beam_kernel(const BeamParams p) {
+__global__ void __launch_bounds__(256, PS::BLOCKS) beam_kernel(const BeamParams p) {
     constexpr int WC = WT ? WT : WMAX;  // parents per round at most
     const int Wr = WT ? WT : p.W;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -787,27 +830,6 @@ __global__ void __launch_bounds__(256, 3) beam_kernel(const BeamParams p) {
                     tS = bS[L - 1];
                     tI = bI[L - 1] & ~(int)EXPANDED;
                 }
-                if (full && cnt > 32) {
-                    // several chunks: drop the ids below the beam first, so that the search for places
-                    // runs over the few that are left
-                    int c2 = 0;
-                    for (int j0 = 0; j0 < cnt; j0 += 32) {
-                        const int j = j0 + lane;
-                        const float s = j < cnt ? wS[j] : 0.f;
-                        const int id = j < cnt ? wI[j] : 0;
-                        const bool keep = j < cnt && key_better(fmaxf(s, -INFINITY), id, tS, tI);
-                        const unsigned bal = __ballot_sync(FULL, keep);
-                        __syncwarp();
-                        if (keep) {
-                            const int o = c2 + __popc(bal & lt);
-                            wI[o] = id;
-                            wS[o] = s;
-                        }
-                        c2 += __popc(bal);
-                    }
-                    cnt = c2;
-                    __syncwarp();
-                }
                 for (int j0 = 0; j0 < cnt; j0 += 32) {
                     const int j = j0 + lane;
                     bool valid = false;
@@ -899,32 +921,10 @@ __global__ void __launch_bounds__(256, 3) beam_kernel(const BeamParams p) {
                             ranks += (unsigned)rank;
                         }
                         if (Wr == 1 || __reduce_add_sync(FULL, ranks) == (unsigned)(cv * (cv - 1) / 2)) break;
-                        int cv2 = 0;
-                        for (int j0 = 0; j0 < cv; j0 += 32) {
-                            const int j = j0 + lane;
-                            bool keep = j < cv;
-                            float s = 0.f;
-                            int id = 0, pb = 0;
-                            if (keep) {
-                                s = cS[j];
-                                id = cI[j];
-                                pb = vPB[j] & 0xffff;
-                                // copies before j: kept ones (already compacted) or of this chunk
-                                for (int u = 0; u < cv2; ++u) keep &= cI[u] != id;
-                                for (int u = j0; u < j; ++u) keep &= cI[u] != id;
-                            }
-                            const unsigned bal = __ballot_sync(FULL, keep);
-                            __syncwarp();
-                            if (keep) {
-                                const int o = cv2 + __popc(bal & lt);
-                                cI[o] = id;
-                                cS[o] = s;
-                                vPB[o] = pb;
-                            }
-                            cv2 += __popc(bal);
-                            __syncwarp();
-                        }
-                        cv = cv2;
+                        if constexpr (PS::COPIES_APART)
+                            cv = drop_copies_apart(cI, cS, vPB, cv, lane);
+                        else
+                            cv = drop_copies(cI, cS, vPB, cv, lane);
                     }
                     __syncwarp();
                     // Merge in place, last 32 places first: a place that no candidate takes holds the beam
