@@ -787,8 +787,12 @@ int build_graph_impl(lv_index *idx, int R, int Lb, float alpha, int passes, int 
             // most targets gain a few edges: the pools of those with at most 32 sources fit many blocks on an
             // SM; the rest (a target may receive many reverse edges in one batch) take a second launch.  The
             // line is drawn on the sources alone, which the first launch does not change: a list it rewrote
-            // must not be taken a second time
-            const int small = std::min(R + 32, PMAX1);
+            // must not be taken a second time.  Where the largest pool is small, one launch takes all: the second
+            // one's blocks cost more to start than the occupancy gives (50,000 nodes of 24 codes, R = 16, pools of
+            // 20 KB: 7.97 ms with two launches, 7.26 with one; 64 codes, R = 32, 36 KB: 13.8 and 13.3; 64 codes,
+            // R = 64, 48 KB: equal; 128 codes, R = 32, 61 KB: 14.8 and 15.1; 160 codes, R = 64, 97 KB: 21.7 and 24.1).
+            const bool one = prune_smem(PMAX1, prune_slot(PMAX1, idx->pg.code_chunks, idx->metric)) <= 40 * 1024;
+            const int small = one ? PMAX1 : std::min(R + 32, PMAX1);
             for (int tier = 0; tier < (small < PMAX1 ? 2 : 1) && !rc; ++tier) {
                 PruneParams pr = pp;
                 pr.PMAX = tier ? PMAX1 : small;
