@@ -1,12 +1,12 @@
 // Rerank kernel (Sec. 2 "Search": the final candidates of the primary search are rescored
 // with the full-dimensional LVQ-8 or FP16 secondary vectors against the unreduced query, and the
 // best k are kept).  The beam kernel hands over the top-r ids of every query (BeamParams::cand);
-// here a block of four warps takes one query.
+// here a block of four warps (two for long FP16 records) takes one query.
 //
 // Bound by the random reads of the secondary records (r x about D bytes per query).  A record
 // goes through a shared-memory ring by cp.async.bulk, one copy per record, RR_GROUP records to a
 // stage, so a warp keeps two stages in flight without holding them in registers.  The warps of a
-// block share a query's candidates (groups w, w + 4, ...) and its byte limbs: the set-up and the
+// block share a query's candidates (group w, w + warps, ...) and its byte limbs: the set-up and the
 // top-k of one query then hide behind the copies of the other blocks of the SM.
 // 152 candidates of 784 bytes per query from a 1M-row store, L2 flushed (time, share of the copy
 // bandwidth): 10,000 queries 213 us (82 %), 3,069 86 us (63 %), 100 20 us; with one warp per query
@@ -19,7 +19,6 @@
 
 namespace lv {
 
-constexpr int RR_WARPS = 4;   // warps of a block, all on one query
 constexpr int RR_GROUP = 4;   // records of a stage (their four sums share one reduction)
 constexpr int RR_STAGES = 2;  // ring stages of a warp
 constexpr uint32_t RR_TRY_NS = 1000000;  // longest suspension of one try of a wait
@@ -55,14 +54,15 @@ struct RerankParams {
 // l + 32 (D <= 1008).
 template <bool L2 = false>
 struct SecIntScorer {
+    static constexpr int WARPS = 4;  // of a block, all on one query
     static constexpr int NCW = 2;
     uint4 qh[NCW], qm[NCW], ql[NCW];
     float c0, s0, scale;
     int CH;
 
-    static __host__ __device__ int query_bytes(int chunks) { return 3 * 16 * chunks; }
+    static constexpr __host__ __device__ int query_bytes(int chunks) { return 3 * 16 * chunks; }
 
-    // Each warp reads the whole query and forms the constants in its lanes' fixed order; the RR_WARPS warps
+    // Each warp reads the whole query and forms the constants in its lanes' fixed order; the WARPS warps
     // share the limbs: byte j of the limb arrays h, m, l belongs to entry j, that is to code j of a
     // record.  Loads go out 16 at a time; the loops stay rolled beyond that, since a small batch
     // runs this code once per SM and pays for every instruction line it fetches.
@@ -99,7 +99,7 @@ struct SecIntScorer {
         scale = amax > 0.f ? amax / 8388607.0f : 1.0f;
         const float inv = amax > 0.f ? 8388607.0f / amax : 0.f;
 #pragma unroll 4
-        for (int j = lane + 32 * wid; j < 16 * CH; j += 32 * RR_WARPS) {  // entries past D are zero
+        for (int j = lane + 32 * wid; j < 16 * CH; j += 32 * WARPS) {  // entries past D are zero
             int qv = j < p.D ? __float2int_rn(__ldg(q + j) * inv) : 0;
             qv = max(-8388607, min(8388607, qv));
             qsm[j] = (unsigned char)(qv >> 16);
@@ -156,15 +156,19 @@ struct SecIntScorer {
 // float32.
 template <int NCW, bool L2 = false>
 struct Fp16SecScorer {
+    // Above 256 dimensions two warps a block: records of 1.5 KB leave an SM four blocks of four warps, too few
+    // queries at once where r is small.  200k x 768, r = 20 / 64 / 152, whole searches against four warps: 2000
+    // queries 1.03 / 1.03 / 1.05 times the speed, 20,000 1.09 / 1.05 / 1.02; up to 256 dimensions equal.
+    static constexpr int WARPS = NCW > 1 ? 2 : 4;
     float q[NCW][8];
     int CH;
 
-    static __host__ __device__ int query_bytes(int chunks) { return 32 * chunks; }
+    static constexpr __host__ __device__ int query_bytes(int chunks) { return 32 * chunks; }
 
     __device__ __forceinline__ void setup(const float *qrow, const RerankParams &p, unsigned char *qsm) {
         CH = p.sec_chunks;
         float *dst = reinterpret_cast<float *>(qsm);
-        for (int j = threadIdx.x; j < 8 * CH; j += 32 * RR_WARPS) dst[j] = j < p.D ? qrow[j] : 0.f;
+        for (int j = threadIdx.x; j < 8 * CH; j += 32 * WARPS) dst[j] = j < p.D ? qrow[j] : 0.f;
     }
 
     __device__ __forceinline__ void load(const unsigned char *qsm, int lane) {
@@ -235,7 +239,7 @@ constexpr int TOPK_ROUNDS = 32;  // up to this k: rounds of a warp maximum; abov
 // The best k of n entries by (score desc, id asc) into oid / osc[0 .. min(k, n)).  key[t] holds the
 // order of entry t, score above id; S its score.  Small k: one warp, a round per result -- two redux
 // instructions for the maximum, its entry cleared.  Larger k: every thread ranks its entries against
-// all (n^2 / (32 RR_WARPS) comparisons a thread, independent of k).
+// all (n^2 / blockDim.x comparisons a thread, independent of k).
 __device__ __forceinline__ void block_topk(unsigned long long *key, const float *S, int n, int k, int32_t *oid,
                                            float *osc) {
     const int tid = threadIdx.x, lane = tid & 31;
@@ -265,7 +269,7 @@ __device__ __forceinline__ void block_topk(unsigned long long *key, const float 
         }
         return;
     }
-    for (int t = tid; t < n; t += 32 * RR_WARPS) {
+    for (int t = tid; t < n; t += (int)blockDim.x) {
         const unsigned long long mine = key[t];
         int rank = 0;
         for (int u = 0; u < n; ++u) rank += key[u] > mine || (key[u] == mine && u < t) ? 1 : 0;
@@ -277,9 +281,10 @@ __device__ __forceinline__ void block_topk(unsigned long long *key, const float 
 }
 
 template <class SS>
-__global__ void __launch_bounds__(32 * RR_WARPS) rerank_kernel(const RerankParams p) {
+__global__ void __launch_bounds__(32 * SS::WARPS) rerank_kernel(const RerankParams p) {
+    constexpr int W = SS::WARPS;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ uint64_t bars[RR_WARPS][RR_STAGES];
+    __shared__ uint64_t bars[W][RR_STAGES];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int64_t qi = blockIdx.x;
     int k = p.desc ? p.desc[qi].x : p.uni.x;
@@ -287,7 +292,7 @@ __global__ void __launch_bounds__(32 * RR_WARPS) rerank_kernel(const RerankParam
 
     const int ring = RR_STAGES * RR_GROUP * p.rec_bytes;  // of one warp
     unsigned char *const my = smem_raw + (size_t)wid * ring;
-    unsigned char *const qsm = smem_raw + (size_t)RR_WARPS * ring;
+    unsigned char *const qsm = smem_raw + (size_t)W * ring;
     unsigned long long *const rK = reinterpret_cast<unsigned long long *>(qsm + SS::query_bytes(p.sec_chunks));
     float *const rS = reinterpret_cast<float *>(rK + p.ldc);
     int *const rI = reinterpret_cast<int *>(rS + p.ldc);
@@ -298,15 +303,15 @@ __global__ void __launch_bounds__(32 * RR_WARPS) rerank_kernel(const RerankParam
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     const int32_t *cd = p.cand + qi * p.ldc;
-    for (int t = tid; t < p.ldc; t += 32 * RR_WARPS) rI[t] = cd[t];  // with the count in flight; the first nr are used
+    for (int t = tid; t < p.ldc; t += 32 * W) rI[t] = cd[t];  // with the count in flight; the first nr are used
     const int nr = min(p.cand_n[qi], p.ldc);
     if (nr < 0) return;  // the whole block
     __syncthreads();
-    // group i of this warp: candidates RR_GROUP (wid + RR_WARPS i) .. + RR_GROUP - 1
+    // group i of this warp: candidates RR_GROUP (wid + W i) .. + RR_GROUP - 1
     const int groups = (nr + RR_GROUP - 1) / RR_GROUP;
-    const int mine = wid < groups ? (groups - wid + RR_WARPS - 1) / RR_WARPS : 0;
+    const int mine = wid < groups ? (groups - wid + W - 1) / W : 0;
     auto issue = [&](int i) {
-        const int b = RR_GROUP * (wid + RR_WARPS * i), cnt = min(RR_GROUP, nr - b), s = i % RR_STAGES;
+        const int b = RR_GROUP * (wid + W * i), cnt = min(RR_GROUP, nr - b), s = i % RR_STAGES;
         if (lane == 0)
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(rr_smem(bar + s)),
                          "r"((uint32_t)(cnt * p.rec_bytes))
@@ -326,7 +331,7 @@ __global__ void __launch_bounds__(32 * RR_WARPS) rerank_kernel(const RerankParam
     sc.load(qsm, lane);
     int i = 0;
     for (; i < mine; ++i) {
-        const int b = RR_GROUP * (wid + RR_WARPS * i), s = i % RR_STAGES;
+        const int b = RR_GROUP * (wid + W * i), s = i % RR_STAGES;
         if (!__all_sync(FULL, rr_wait(bar + s, (uint32_t)(i / RR_STAGES) & 1u, p.tries))) break;
         const unsigned char *rec = my + (size_t)s * RR_GROUP * p.rec_bytes;
         // sums over the warp of the four records: the halves of a lane pair each take on two records,
@@ -360,23 +365,25 @@ __global__ void __launch_bounds__(32 * RR_WARPS) rerank_kernel(const RerankParam
     int32_t *oid = p.ids + qi * p.ldo;
     float *osc = p.scores + qi * p.ldo;
     block_topk(rK, rS, n, k, oid, osc);
-    for (int t = min(k, n) + tid; t < p.ldo; t += 32 * RR_WARPS) {
+    for (int t = min(k, n) + tid; t < p.ldo; t += 32 * W) {
         oid[t] = -1;
         osc[t] = -INFINITY;
     }
 }
 
-// the largest case: FP16 records of 1024 dimensions and L = LCAP_MAX
-constexpr int RR_SMEM_MAX = RR_WARPS * RR_STAGES * RR_GROUP * 2048 + 32 * 128 + 16 * LCAP_MAX;
+// bytes of a block's ring, query and candidates; without more than 48 KB no limit has to be raised (see allow_smem)
+template <class SS>
+static constexpr size_t rerank_smem(int rec_bytes, int chunks, int ldc) {
+    return (size_t)SS::WARPS * RR_STAGES * RR_GROUP * rec_bytes + SS::query_bytes(chunks) + 16 * (size_t)ldc;
+}
+static_assert(rerank_smem<SecIntScorer<true>>(1024, 63, LCAP_MAX) <= 48 * 1024, "LVQ-8, 64 chunks");
+static_assert(rerank_smem<Fp16SecScorer<4>>(2048, 128, LCAP_MAX) <= 48 * 1024, "FP16, 1024 dimensions");
+static_assert(rerank_smem<Fp16SecScorer<1>>(512, 32, LCAP_MAX) <= 48 * 1024, "FP16, 256 dimensions, four warps");
 
 template <class SS>
 static int go_rerank(const RerankParams &p, cudaStream_t st) {
-    const size_t smem = (size_t)RR_WARPS * RR_STAGES * RR_GROUP * p.rec_bytes + SS::query_bytes(p.sec_chunks) +
-                        16 * (size_t)p.ldc;
-    // one limit for all sizes (see allow_smem), and none to set where every kernel may have as much
-    if (smem > 48 * 1024)
-        LV_CUDA(cudaFuncSetAttribute(rerank_kernel<SS>, cudaFuncAttributeMaxDynamicSharedMemorySize, RR_SMEM_MAX));
-    rerank_kernel<SS><<<(unsigned)p.m, 32 * RR_WARPS, smem, st>>>(p);
+    const size_t smem = rerank_smem<SS>(p.rec_bytes, p.sec_chunks, p.ldc);
+    rerank_kernel<SS><<<(unsigned)p.m, 32 * SS::WARPS, smem, st>>>(p);
     LV_CHECK_LAUNCH("rerank_kernel");
     return LV_OK;
 }
