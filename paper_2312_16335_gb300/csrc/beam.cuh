@@ -575,8 +575,8 @@ __device__ __forceinline__ bool bucket_tag_free(const uint4 v, unsigned tag, int
 
 // Keeps the first copy of every id among the cv candidates of a round, in order; returns their number (one
 // warp).  Rare, and called out of line by the float32 scorers, whose queries and records leave no registers
-// for it: inlined it cost the walks of 768-dimensional records at width 2 13 to 16 % (12 bytes of spills and a
-// slower schedule for 0), while the LVQ scorers lose 1 % by the call.
+// for it: inlined, it lengthened walks over 768-dimensional records at width 2 by 13 to 16 % (100 queries,
+// 300k rows, L = 20: 597 us, out of line 498), while the LVQ scorers lose 1 % by the call.
 __device__ __forceinline__ int drop_copies(int *cI, float *cS, int *vPB, int cv, int lane) {
     const unsigned lt = (1u << lane) - 1u;
     int cv2 = 0;
